@@ -2,8 +2,8 @@
 
 Each translation unit compiles in its own nvcc process, in parallel; the objects
 are linked with ``nvcc -shared`` (static CUDA runtime). No cmake. The fused step
-kernel, step_inst.cu, is compiled once per (lattice, storage type), since its
-instantiations dominate the build time.
+kernel, step_inst.cu, is compiled once per part of each (lattice, storage type),
+since its instantiations dominate the build time.
 """
 from __future__ import annotations
 
@@ -33,8 +33,10 @@ COMMON = ARCH + ["-O3", "-lineinfo", "-std=c++20", "-Xcompiler", "-fPIC", "--exp
                  "-Xptxas", "--fmad=false", "-I", INCLUDE]
 # per-file extra flags: the geometry kernels round like the plain FP64 definitions
 EXTRA = {"geometry.cu": ["-fmad=false"]}
-# step_inst.cu: one object per (lattice, storage type)
+# step_inst.cu: one object per (lattice, storage type) and part (one-node kernels;
+# node pairs and TMA; split and batched step)
 STEP_INSTANCES = [(lat, sto) for lat in ("D2Q9", "D3Q19", "D3Q27") for sto in ("double", "float", "__half", "__nv_bfloat16")]
+STEP_PARTS = (0, 1, 2)
 
 
 def _nvcc():
@@ -72,13 +74,14 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     jobs = []
     for src in srcs:
         if src == "step_inst.cu":
-            for lat, sto in STEP_INSTANCES:
-                jobs.append((src, [f"-DLBM_STEP_LATTICE={lat}", f"-DLBM_STEP_STORE={sto}"],
-                             f"step_{lat}_{sto.strip('_')}.o"))
+            for part in STEP_PARTS:
+                for lat, sto in STEP_INSTANCES:
+                    jobs.append((src, [f"-DLBM_STEP_PART={part}", f"-DLBM_STEP_LATTICE={lat}",
+                                       f"-DLBM_STEP_STORE={sto}"], f"step_{lat}_{sto.strip('_')}_{part}.o"))
         else:
             jobs.append((src, EXTRA.get(src, []), src.replace(".cu", ".o")))
-    # the slowest units first, so that they overlap with the rest
-    jobs.sort(key=lambda j: j[0] != "step_inst.cu")
+    # the slowest units first, so that they overlap with the rest: the step kernels, by number of directions
+    jobs.sort(key=lambda j: (j[0] != "step_inst.cu", "D3Q27" not in j[2], "D3Q19" not in j[2], "double" in j[2]))
 
     def compile_one(job):
         src, flags, name = job

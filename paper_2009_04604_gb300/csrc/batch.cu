@@ -49,63 +49,20 @@ static int bfail(lbm_batch b, int code, const std::string &msg) {
                    std::string(#call) + ": " + cudaGetErrorString(e_));                          \
   } while (0)
 
-template <class L, typename S, typename M, int MINB, int PHYS>
-static cudaError_t batch_class(const lbm_batch_s *b, int parity) {
-  const long long n = b->cls_count[PHYS];
-  if (n == 0) return cudaSuccess;
-  const dim3 block(b->bx, b->by, 1);
-  const unsigned grid = (unsigned)((n + b->T - 1) / b->T);
-  k_step_batch<L, S, M, MINB, PHYS><<<grid, block, 0, b->stream>>>(b->entries, b->tiles + b->cls_first[PHYS],
-                                                                    (int)n, b->T, parity);
-  return cudaGetLastError();
-}
-
-template <class L, typename S, typename M, int MINB>
-static cudaError_t batch_variant(const lbm_batch_s *b, int parity) {
-  cudaError_t e = batch_class<L, S, M, MINB, 0>(b, parity);
-  if (e == cudaSuccess) e = batch_class<L, S, M, MINB, PH_FORCE>(b, parity);
-  if (e == cudaSuccess) e = batch_class<L, S, M, MINB, PH_TRT>(b, parity);
-  if (e == cudaSuccess) e = batch_class<L, S, M, MINB, PH_FORCE | PH_TRT>(b, parity);
-  return e;
-}
-
-template <class L, typename S, typename M>
-static cudaError_t batch_launch_t(const lbm_batch_s *b, int parity) {
-  if constexpr (sizeof(M) == 8) {
-    return batch_variant<L, S, M, 1>(b, parity);
-  } else {
-    switch (b->variant) {
-      case 1: return batch_variant<L, S, M, 2>(b, parity);
-      case 2: return batch_variant<L, S, M, 3>(b, parity);
-      case 3: return batch_variant<L, S, M, 4>(b, parity);
-      default: return batch_variant<L, S, M, 1>(b, parity);
-    }
-  }
-}
-
+// One step of every physics class present in the batch.
 static cudaError_t batch_launch(const lbm_batch_s *b, int parity) {
-  if (b->lattice == LBM_D2Q9) {
-    switch (b->dtype) {
-      case LBM_F64: return batch_launch_t<D2Q9, double, double>(b, parity);
-      case LBM_F32: return batch_launch_t<D2Q9, float, float>(b, parity);
-      case LBM_F16: return batch_launch_t<D2Q9, __half, float>(b, parity);
-      default: return batch_launch_t<D2Q9, __nv_bfloat16, float>(b, parity);
-    }
+  Launch l;
+  l.block = dim3(b->bx, b->by, 1);
+  l.stream = b->stream;
+  for (int c = 0; c < 4; ++c) {
+    const long long n = b->cls_count[c];
+    if (n == 0) continue;
+    l.grid = dim3((unsigned)((n + b->T - 1) / b->T));
+    cudaError_t e = launch_step_batch(b->lattice, b->dtype, b->variant, c, b->entries, b->tiles + b->cls_first[c],
+                                      (int)n, b->T, parity, l);
+    if (e != cudaSuccess) return e;
   }
-  if (b->lattice == LBM_D3Q27) {
-    switch (b->dtype) {
-      case LBM_F64: return batch_launch_t<D3Q27, double, double>(b, parity);
-      case LBM_F32: return batch_launch_t<D3Q27, float, float>(b, parity);
-      case LBM_F16: return batch_launch_t<D3Q27, __half, float>(b, parity);
-      default: return batch_launch_t<D3Q27, __nv_bfloat16, float>(b, parity);
-    }
-  }
-  switch (b->dtype) {
-    case LBM_F64: return batch_launch_t<D3Q19, double, double>(b, parity);
-    case LBM_F32: return batch_launch_t<D3Q19, float, float>(b, parity);
-    case LBM_F16: return batch_launch_t<D3Q19, __half, float>(b, parity);
-    default: return batch_launch_t<D3Q19, __nv_bfloat16, float>(b, parity);
-  }
+  return cudaSuccess;
 }
 
 static void drop_batch_graphs(lbm_batch b) {

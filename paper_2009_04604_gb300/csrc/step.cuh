@@ -1,10 +1,11 @@
 // step.cuh -- launch of the fused step kernel for one (lattice, storage type).
 //
 // The step kernel has many instantiations (register budget, node pairs, force
-// path, the TMA-staged kernel). They are compiled in one translation unit per
-// (lattice, storage type), step_inst.cu built once for each pair, so that the
-// build runs them in parallel. kernels.cu dispatches to the explicit
-// instantiations of launch_step_ls and prepare_step_tma_ls.
+// path, the TMA-staged kernel). They are compiled in three translation units per
+// (lattice, storage type), step_inst.cu built once for each part of each pair, so
+// that the build runs them in parallel: the one-node kernels (launch_one_ls), the
+// node pairs and the TMA-staged kernel (launch_wide_ls), the split step and the
+// batched step (launch_split_ls, launch_batch_ls). kernels.cu dispatches to them.
 #pragma once
 
 #include "kernels.cuh"
@@ -110,17 +111,31 @@ cudaError_t tma_launch(const View &v, const void *fin, void *fout, const Launch 
 template <typename S> struct MathOf { using T = float; };
 template <> struct MathOf<double> { using T = double; };
 
+// Register budgets: variants 0..2 share one kernel. At 80 registers (3 resident
+// 256-thread blocks) no one-node kernel of any lattice spills, so the looser
+// budgets of variants 0 and 1 would only lower the number of resident warps.
+// Variants 5 and 6 share one in the same way (two blocks, 128 registers).
 template <class L, typename S>
-cudaError_t launch_step_ls(int variant, const View &v, const void *fin, void *fout, const Launch &l,
-                           const Launch *lb) {
+cudaError_t launch_one_ls(int variant, const View &v, const void *fin, void *fout, const Launch &l) {
   using M = typename MathOf<S>::T;
   if constexpr (sizeof(M) == 8) {
     return step_variant<L, S, M, 1>(v, fin, fout, l);  // FP64: one register budget
   } else {
-    if (variant == 9) return split_variant<L, S, M, 6>(v, fin, fout, l, lb);
-    if (variant == 10) return split_variant<L, S, M, 5>(v, fin, fout, l, lb);
-    if (variant == 11) return step_variant<L, S, M, 5>(v, fin, fout, l);
-    if (variant == 12) return step_variant<L, S, M, 6>(v, fin, fout, l);
+    switch (variant) {
+      case 3: return step_variant<L, S, M, 4>(v, fin, fout, l);
+      case 11: return step_variant<L, S, M, 5>(v, fin, fout, l);
+      case 12: return step_variant<L, S, M, 6>(v, fin, fout, l);
+      default: return step_variant<L, S, M, 3>(v, fin, fout, l);
+    }
+  }
+}
+
+template <class L, typename S>
+cudaError_t launch_wide_ls(int variant, const View &v, const void *fin, void *fout, const Launch &l) {
+  using M = typename MathOf<S>::T;
+  if constexpr (sizeof(M) == 8) {
+    return cudaErrorInvalidValue;
+  } else {
     if (variant == 4) {
       switch (phys_of(v)) {
         case PH_FORCE: return tma_launch<L, S, M, PH_FORCE>(v, fin, fout, l);
@@ -129,17 +144,44 @@ cudaError_t launch_step_ls(int variant, const View &v, const void *fin, void *fo
         default: return tma_launch<L, S, M, 0>(v, fin, fout, l);
       }
     }
-    switch (variant) {
-      case 1: return step_variant<L, S, M, 2>(v, fin, fout, l);
-      case 2: return step_variant<L, S, M, 3>(v, fin, fout, l);
-      case 3: return step_variant<L, S, M, 4>(v, fin, fout, l);
-      case 5: return step_variant<L, S, M, 1, true>(v, fin, fout, l);
-      case 6: return step_variant<L, S, M, 2, true>(v, fin, fout, l);
-      case 7: return step_variant<L, S, M, 3, true>(v, fin, fout, l);
-      case 8: return step_variant<L, S, M, 7, true, 128>(v, fin, fout, l);
-      default: return step_variant<L, S, M, 1>(v, fin, fout, l);
-    }
+    if (variant == 7) return step_variant<L, S, M, 3, true>(v, fin, fout, l);
+    if (variant == 8) return step_variant<L, S, M, 7, true, 128>(v, fin, fout, l);
+    return step_variant<L, S, M, 2, true>(v, fin, fout, l);
   }
+}
+
+template <class L, typename S>
+cudaError_t launch_split_ls(int variant, const View &v, const void *fin, void *fout, const Launch &l,
+                            const Launch *lb) {
+  using M = typename MathOf<S>::T;
+  if constexpr (sizeof(M) == 8) return cudaErrorInvalidValue;
+  else if (variant == 9) return split_variant<L, S, M, 6>(v, fin, fout, l, lb);
+  else return split_variant<L, S, M, 5>(v, fin, fout, l, lb);
+}
+
+// Batched step of the tiles of one physics class (l.grid.x blocks); variant 0..2: 80
+// registers, 3: 64.
+template <class L, typename S, typename M, int MINB>
+cudaError_t batch_variant(int phys, const BatchEntry *e, const int4 *tiles, int n, int T, int parity,
+                          const Launch &l) {
+  switch (phys) {
+    case PH_FORCE: k_step_batch<L, S, M, MINB, PH_FORCE><<<l.grid, l.block, 0, l.stream>>>(e, tiles, n, T, parity); break;
+    case PH_TRT: k_step_batch<L, S, M, MINB, PH_TRT><<<l.grid, l.block, 0, l.stream>>>(e, tiles, n, T, parity); break;
+    case PH_FORCE | PH_TRT:
+      k_step_batch<L, S, M, MINB, PH_FORCE | PH_TRT><<<l.grid, l.block, 0, l.stream>>>(e, tiles, n, T, parity);
+      break;
+    default: k_step_batch<L, S, M, MINB, 0><<<l.grid, l.block, 0, l.stream>>>(e, tiles, n, T, parity); break;
+  }
+  return cudaGetLastError();
+}
+
+template <class L, typename S>
+cudaError_t launch_batch_ls(int variant, int phys, const BatchEntry *e, const int4 *tiles, int n, int T,
+                            int parity, const Launch &l) {
+  using M = typename MathOf<S>::T;
+  if constexpr (sizeof(M) == 8) return batch_variant<L, S, M, 1>(phys, e, tiles, n, T, parity, l);
+  else if (variant == 3) return batch_variant<L, S, M, 4>(phys, e, tiles, n, T, parity, l);
+  else return batch_variant<L, S, M, 3>(phys, e, tiles, n, T, parity, l);
 }
 
 template <class L, typename S>
@@ -162,9 +204,19 @@ cudaError_t prepare_step_tma_ls(int phys, int bx, int by, long long ntiles, int 
   X(D3Q19, double) X(D3Q19, float) X(D3Q19, __half) X(D3Q19, __nv_bfloat16) \
   X(D3Q27, double) X(D3Q27, float) X(D3Q27, __half) X(D3Q27, __nv_bfloat16)
 
-#define LBM_STEP_DECLARE(Lat, Sto)                                                                  \
-  extern template cudaError_t launch_step_ls<Lat, Sto>(int, const View &, const void *, void *,    \
-                                                       const Launch &, const Launch *);           \
-  extern template cudaError_t prepare_step_tma_ls<Lat, Sto>(int, int, int, long long, int *, int *);
+#define LBM_STEP_PART0(X, Lat, Sto) \
+  X template cudaError_t launch_one_ls<Lat, Sto>(int, const View &, const void *, void *, const Launch &);
+#define LBM_STEP_PART1(X, Lat, Sto)                                                                       \
+  X template cudaError_t launch_wide_ls<Lat, Sto>(int, const View &, const void *, void *, const Launch &); \
+  X template cudaError_t prepare_step_tma_ls<Lat, Sto>(int, int, int, long long, int *, int *);
+#define LBM_STEP_PART2(X, Lat, Sto)                                                              \
+  X template cudaError_t launch_split_ls<Lat, Sto>(int, const View &, const void *, void *, const Launch &, \
+                                                   const Launch *);                              \
+  X template cudaError_t launch_batch_ls<Lat, Sto>(int, int, const BatchEntry *, const int4 *, int, int, int, \
+                                                   const Launch &);
+#define LBM_STEP_DECLARE(Lat, Sto)      \
+  LBM_STEP_PART0(extern, Lat, Sto)      \
+  LBM_STEP_PART1(extern, Lat, Sto)      \
+  LBM_STEP_PART2(extern, Lat, Sto)
 
 }  // namespace lbm
