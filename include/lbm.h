@@ -389,16 +389,24 @@ int lbm_set_debug_limit(lbm_handle h, long long elements);
  *     block of the boundary kernel takes one boundary-record tile).
  * FP64 storage accepts variant 0 only, and on D3Q27 at most 128 threads per block
  * (27 x 256 doubles of boundary staging would exceed the static shared memory).
- * The default is the widest bx <= 128 that divides the row, by = 256/bx (128/bx
- * for FP64 on D3Q27), variant 0, tiles 4. LBM_ERR_ARG for an invalid
- * configuration. */
+ * Variants 0..3, 11 and 12 step in bulk tiles where the rule is ELIBB-F or -FQ with
+ * the bounce-back wall estimate and the geometry has no thin shell: one kernel whose
+ * grid is the lattice and whose warps also evaluate the links of scattered boundary
+ * nodes, with the boundary tiles of flat walls and of a moving body in a second kernel
+ * beside it, as in the split step. `tiles` then counts tiles one above the other.
+ * The results are the same. Variants 0 and 1 share the register budget of variant 2,
+ * variant 5 that of variant 6.
+ * Until this call or lbm_autotune the library chooses by size, type and rule: blocks
+ * of 32 x 4 nodes (FP64: 32 x 1 or 32 x 2) in variant 11 or 3 (FP64: 0), one
+ * tile per block or, on large lattices, two. lbm_get_launch returns what is in use.
+ * LBM_ERR_ARG for an invalid configuration. */
 int lbm_set_launch(lbm_handle h, int bx, int by, int variant, int tiles);
 int lbm_get_launch(lbm_handle h, int *bx, int *by, int *variant, int *tiles);
 
 /* Autotuner: runs `steps` steps with each candidate configuration and keeps the
  * fastest. The candidates are 128- and 256-thread blocks, every admissible bx,
- * every register variant, and 1, 2 or 4 tiles per block. Each is timed with
- * CUDA events. The simulation advances by every trial step. Writes the chosen
+ * every variant with a kernel of its own, and 1, 2 or 4 tiles per block. Each is
+ * timed with CUDA events. The simulation advances by every trial step. Writes the chosen
  * configuration and its time per step in ms; any output may be NULL.
  * Synchronises the stream. */
 int lbm_autotune(lbm_handle h, int steps, int *bx, int *by, int *variant, int *tiles,

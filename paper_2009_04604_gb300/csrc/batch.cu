@@ -1,10 +1,10 @@
 // batch.cu -- batched stepping of many independent simulations (lbm_batch_*).
 //
-// One launch per step and physics class (body force on or off, BGK or TRT; a
-// batch of like simulations has one class) advances every simulation of the
-// batch. Its blocks run the tiles of the class's simulations, one simulation
-// after another, each one's table plane-interleaved as in the single-simulation
-// step. The steps replay from captured CUDA graphs.
+// Every step takes one launch per physics class (body force on or off, BGK or TRT; a
+// batch of like simulations has one class) for the bulk tiles of all simulations that
+// step in bulk (lbm_sim::fused), with one launch for their boundary tiles beside it on
+// a second stream of the batch, and one launch per class for the tiles of the others.
+// The steps replay from captured CUDA graphs.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,7 +26,13 @@ struct lbm_batch_s {
   BatchEntry *entries = nullptr;
   int4 *tiles = nullptr;
   long long ntiles = 0;
-  long long cls_first[4] = {0, 0, 0, 0}, cls_count[4] = {0, 0, 0, 0};  // tile range per physics class
+  struct Range {
+    long long first = 0, count = 0;
+    int smem = 0;  // dynamic shared memory of a block
+  };
+  Range bulk[4], rest[4], boundary;  // tiles by physics class: bulk tiles, the other simulations'; boundary tiles
+  cudaStream_t aux = nullptr;        // the boundary tiles' stream, forked and joined around every step
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int bx = 32, by = 4, variant = 3, T = 1;
   bool tiles_ok = false;
   int parity = 0;  // batch steps taken since the entries were built, mod 2
@@ -49,20 +55,33 @@ static int bfail(lbm_batch b, int code, const std::string &msg) {
                    std::string(#call) + ": " + cudaGetErrorString(e_));                          \
   } while (0)
 
-// One step of every physics class present in the batch.
+// One step of the whole batch. The kernels of a step only read the buffers of one
+// parity and write disjoint slots of the other, so that they need no order.
 static cudaError_t batch_launch(const lbm_batch_s *b, int parity) {
   Launch l;
   l.block = dim3(b->bx, b->by, 1);
-  l.stream = b->stream;
-  for (int c = 0; c < 4; ++c) {
-    const long long n = b->cls_count[c];
-    if (n == 0) continue;
-    l.grid = dim3((unsigned)((n + b->T - 1) / b->T));
-    cudaError_t e = launch_step_batch(b->lattice, b->dtype, b->variant, c, b->entries, b->tiles + b->cls_first[c],
-                                      (int)n, b->T, parity, l);
-    if (e != cudaSuccess) return e;
+  const auto run = [&](int kind, int phys, const lbm_batch_s::Range &r, int T, cudaStream_t st) {
+    if (r.count == 0) return cudaSuccess;
+    l.stream = st;
+    l.smem = r.smem;
+    l.grid = dim3((unsigned)((r.count + T - 1) / T));
+    return launch_step_batch(b->lattice, b->dtype, b->variant, kind, phys, b->entries, b->tiles + r.first,
+                             (int)r.count, T, parity, l);
+  };
+  cudaError_t e = cudaSuccess;
+  const bool fork = b->boundary.count > 0;
+  if (fork) {
+    e = cudaEventRecord(b->ev_fork, b->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->aux, b->ev_fork, 0);
+    if (e == cudaSuccess) e = run(kBatchBoundary, 0, b->boundary, 1, b->aux);
   }
-  return cudaSuccess;
+  for (int c = 0; c < 4 && e == cudaSuccess; ++c) e = run(kBatchBulk, c, b->bulk[c], b->T, b->stream);
+  for (int c = 0; c < 4 && e == cudaSuccess; ++c) e = run(kBatchStep, c, b->rest[c], b->T, b->stream);
+  if (fork && e == cudaSuccess) {
+    e = cudaEventRecord(b->ev_join, b->aux);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
+  }
+  return e;
 }
 
 static void drop_batch_graphs(lbm_batch b) {
@@ -79,23 +98,18 @@ static int build_batch(lbm_batch b) {
   b->base_cur.resize(n);
   b->base_ver.resize(n);
   const int tpb = b->bx * b->by;
-  // simulations by physics class, in batch order within a class
-  std::vector<int> order;
-  for (int c = 0; c < 4; ++c)
-    for (int k = 0; k < n; ++k) {
-      const lbm_sim *s = b->sims[k];
-      if (((s->has_force ? PH_FORCE : 0) | (s->collision == LBM_COLL_TRT ? PH_TRT : 0)) == c) order.push_back(k);
-    }
-  for (int c = 0; c < 4; ++c) b->cls_count[c] = 0;
-  for (int k : order) {
+  // The tables one after another: per physics class the bulk tiles and the other
+  // simulations' tiles, in batch order, then the boundary tiles of the former.
+  std::vector<int4> bulk[4], rest[4], bnd;
+  lbm_batch_s::Range rb[4], rr[4], rbnd;
+  for (int k = 0; k < n; ++k) {
     lbm_sim *s = b->sims[k];
     const int c = (s->has_force ? PH_FORCE : 0) | (s->collision == LBM_COLL_TRT ? PH_TRT : 0);
-    if (b->cls_count[c] == 0) b->cls_first[c] = (long long)t.size();
-    const size_t t0 = t.size();
     const int save_bx = s->step_bx, save_var = s->variant;
     s->step_bx = b->bx;        // the view's tile-row count follows the batch's block width
     s->variant = b->variant;   // and its one-node lattice tiles (a simulation may be set to node pairs)
     e[k].v = s->view();
+    const bool fused = s->fused();
     s->step_bx = save_bx;
     s->variant = save_var;
     e[k].v.tiles = nullptr;
@@ -104,20 +118,45 @@ static int build_batch(lbm_batch b) {
     b->base_cur[k] = s->cur;
     b->base_ver[k] = s->version;
     const int gx = s->nxp / b->bx, gy = (s->ny + b->by - 1) / b->by;
-    std::vector<uint32_t> hc(s->np / 32 + 1, 0u);
-    if (s->nb > 0) {
+    std::vector<int4> &lat = fused ? bulk[c] : rest[c], &bt = fused ? bnd : rest[c];
+    lbm_batch_s::Range &rl = fused ? rb[c] : rr[c];
+    if (fused) rl.smem = std::max(rl.smem, s->step_smem(tpb, false, s->nb > 0));
+    else if (s->nb > 0) rl.smem = std::max(rl.smem, s->step_smem(tpb, true, false));
+    std::vector<uint32_t> hc(fused || s->nb == 0 ? 0 : s->np / 32 + 1, 0u);
+    if (!hc.empty()) {
       B_CUDA(b, cudaMemcpyAsync(hc.data(), s->cbase, hc.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, b->stream));
       B_CUDA(b, cudaStreamSynchronize(b->stream));
     }
     const long long pchunks = (long long)s->nxp * s->ny / 32;
     for (int z = 0; z < s->nz; ++z) {
-      for (int i = 0; i < gx * gy; ++i) t.push_back(make_int4(k, z, i, 0));
+      for (int i = 0; i < gx * gy; ++i)
+        lat.push_back(fused ? make_int4(k, z, i % gx, i / gx) : make_int4(k, z, i, 0));
       if (s->nb == 0) continue;
-      const long long r0 = hc[z * pchunks], r1 = hc[(z + 1) * pchunks];
+      const long long r0 = fused ? s->rplane[z] : hc[z * pchunks], r1 = fused ? s->rplane[z + 1] : hc[(z + 1) * pchunks];
       for (long long r = r0; r < r1; r += tpb)
-        t.push_back(make_int4(k, -1, (int)r, (int)std::min<long long>(tpb, r1 - r)));
+        bt.push_back(make_int4(k, -1, (int)r, (int)std::min<long long>(tpb, r1 - r)));
     }
-    b->cls_count[c] += (long long)(t.size() - t0);
+    if (fused && !bnd.empty()) rbnd.smem = std::max(rbnd.smem, s->step_smem(tpb, true, false));
+  }
+  const auto place = [&](const std::vector<int4> &src, lbm_batch_s::Range &r) {
+    r.first = (long long)t.size();
+    r.count = (long long)src.size();
+    t.insert(t.end(), src.begin(), src.end());
+  };
+  for (int c = 0; c < 4; ++c) {
+    place(bulk[c], rb[c]);
+    place(rest[c], rr[c]);
+    b->bulk[c] = rb[c];
+    b->rest[c] = rr[c];
+  }
+  place(bnd, rbnd);
+  b->boundary = rbnd;
+  if (rbnd.count > 0 && !b->aux) {  // highest priority: the boundary blocks start as soon as the step does
+    int lo = 0, hi = 0;
+    B_CUDA(b, cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    B_CUDA(b, cudaStreamCreateWithPriority(&b->aux, cudaStreamNonBlocking, hi));
+    B_CUDA(b, cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
+    B_CUDA(b, cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming));
   }
   drop_batch_graphs(b);
   cudaFree(b->entries);
@@ -190,6 +229,9 @@ extern "C" int lbm_batch_destroy(lbm_batch b) {
   drop_batch_graphs(b);
   cudaFree(b->entries);
   cudaFree(b->tiles);
+  if (b->aux) { cudaStreamSynchronize(b->aux); cudaStreamDestroy(b->aux); }
+  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+  if (b->ev_join) cudaEventDestroy(b->ev_join);
   delete b;
   return LBM_OK;
 }

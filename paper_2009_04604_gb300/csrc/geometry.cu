@@ -406,6 +406,107 @@ __global__ void k_geo_fill(const GeoView g, const uint32_t *__restrict__ cbase,
   rec[rid] = r;
 }
 
+// Links of the boundary nodes by 32-node chunk, one warp per chunk (View::chunk and
+// View::ldesc). The boundary nodes of most chunks are left to the lattice tiles and
+// get F_LINKS. Only the records of chunks with more than kTileRecords boundary nodes
+// are packed for the boundary tiles. Why the line lies there: such a chunk is a piece
+// of a flat wall. Its records gather whole rows and have equally many links, so that a
+// boundary tile does them at full width, while the lattice warp would run five rounds
+// of its link loop one after another (D3Q19 duct, 256 x 128 x 128, at 64 registers:
+// 113 us a step with the walls in boundary tiles, 132 the other way round, FP16 92 and
+// 109). Scattered records are the opposite case: a boundary tile gathers 32 sectors per
+// plane for them and waits for the one with the most links (porous medium of 192^3,
+// FP16: 223 us with all its chunks in the lattice tiles, 285 with none; 150^3 in FP32:
+// 121 and 186). Between 24 and 32 nodes hardly any chunk lies, in either.
+// First (k_geo_lcount) the open links and the packed records are counted per chunk,
+// then, with their exclusive scans, the descriptors and the packed records are
+// written. The wall links of a chunk lie in the link arrays one after another (link0
+// counts them in record order).
+constexpr int kTileRecords = 24;
+
+struct ChunkLinks {
+  Rec r;
+  bool isb, fused;
+  uint32_t open, nw, no, sw, so;  // own open mask; the chunk's wall and open links, and those up to this lane
+};
+
+__device__ __forceinline__ ChunkLinks chunk_links(const View &v, long long n) {
+  ChunkLinks c;
+  const int lane = threadIdx.x & 31;
+  c.r = Rec{0u, 0u, 0u, 0u, 0u};
+  c.isb = (v.flags[n] & 3) == K_FLUID && (v.flags[n] & F_BOUNDARY);
+  const uint32_t bal = __ballot_sync(0xffffffffu, c.isb);
+  if (c.isb) c.r = *record_of(v, n, bal);
+  c.open = c.r.open & ~REC_MOVING;
+  c.sw = __popc(c.r.cut);
+  c.so = __popc(c.open);
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t a = __shfl_up_sync(0xffffffffu, c.sw, o), b = __shfl_up_sync(0xffffffffu, c.so, o);
+    if (lane >= o) { c.sw += a; c.so += b; }
+  }
+  c.nw = __shfl_sync(0xffffffffu, c.sw, 31);
+  c.no = __shfl_sync(0xffffffffu, c.so, 31);
+  c.fused = __popc(bal) <= kTileRecords;
+  return c;
+}
+
+__global__ void k_geo_lcount(const View v, uint32_t *__restrict__ copen, uint32_t *__restrict__ crest) {
+  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= v.np) return;  // whole warps
+  const ChunkLinks c = chunk_links(v, n);
+  const uint32_t bal = __ballot_sync(0xffffffffu, c.isb);
+  if ((threadIdx.x & 31) == 0) {
+    copen[n >> 5] = c.no;
+    crest[n >> 5] = c.fused ? 0u : __popc(bal);
+  }
+}
+
+template <class L>
+__global__ void k_geo_links(const View v, const uint32_t *__restrict__ obase,
+                            const uint32_t *__restrict__ rbase, uint8_t *__restrict__ flags,
+                            uint4 *__restrict__ chunk, uint16_t *__restrict__ ldesc, Rec *__restrict__ rrec,
+                            uint32_t *__restrict__ rrnode) {
+  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= v.np) return;  // whole warps
+  const int lane = threadIdx.x & 31;
+  const ChunkLinks c = chunk_links(v, n);
+  const uint32_t bal = __ballot_sync(0xffffffffu, c.isb);
+  const uint32_t mov = __ballot_sync(0xffffffffu, (c.r.open & REC_MOVING) != 0);
+  const uint32_t li0 = __shfl_sync(0xffffffffu, c.r.link0, bal ? __ffs(bal) - 1 : 0);
+  const uint32_t e0 = (bal ? li0 : 0u) + obase[n >> 5];
+  const int x = (int)(n % v.nxp), y = (int)((n / v.nxp) % v.ny), z = (int)(n / ((long long)v.nxp * v.ny));
+  const uint32_t fbal = __ballot_sync(0xffffffffu, (v.flags[n] & 3) == K_FLUID);
+  const bool fused = c.fused && bal != 0;
+  if (lane == 0) {
+    const bool inside = x > 0 && x + 32 < v.nx && y > 0 && y < v.ny - 1 && (L::D == 2 || (z > 0 && z < v.nz - 1));
+    const uint32_t bits = (fused ? CK_LINKS : 0u) | (fbal == 0 ? CK_IDLE : 0u) |
+                          (fbal == 0xffffffffu && inside ? CK_PLAIN : 0u);
+    chunk[n >> 5] = make_uint4(e0, li0, c.nw | c.no << 10 | (mov ? 1u << 20 : 0u), bits);
+  }
+  if (!c.isb) return;
+  if (!c.fused) {
+    const uint32_t k = rbase[n >> 5] + __popc(bal & ((1u << lane) - 1u));
+    rrec[k] = c.r;
+    rrnode[k] = (uint32_t)n;
+    return;
+  }
+  flags[n] |= F_LINKS;
+  uint32_t ow = e0 + c.sw - __popc(c.r.cut), oo = e0 + c.nw + c.so - __popc(c.open);
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    if ((c.r.cut >> i) & 1u) ldesc[ow++] = link_desc(lane, i);
+    else if ((c.open >> i) & 1u) ldesc[oo++] = link_desc(lane, i);
+  }
+}
+
+// The chunks of a moving body's region look at the flags in every step.
+__global__ void k_move_chunks(const View v, int ox, int oy, int oz, int rx, int ry, int rz, uint4 *__restrict__ chunk) {
+  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= (long long)rx * ry * rz) return;
+  const int x = ox + (int)(r % rx), y = oy + (int)((r / rx) % ry), z = oz + (int)(r / ((long long)rx * ry));
+  chunk[(((long long)z * v.ny + y) * v.nxp + x) >> 5].w &= ~(uint32_t)CK_PLAIN;
+}
+
 cudaError_t launch_amask(int lattice, const View &v, uint32_t *amask, cudaStream_t s) {
   const unsigned blocks = (unsigned)((v.np + 255) / 256);
   if (lattice == 0) k_geo_amask<D2Q9><<<blocks, 256, 0, s>>>(v, amask);
@@ -454,6 +555,45 @@ void exclusive_scan(uint32_t *a, long long n, uint32_t *tot, uint32_t *total, cu
   k_scan_block<<<(unsigned)nblk, 1024, 0, st>>>(a, n, tot);
   k_scan_totals<<<1, 1, 0, st>>>(tot, nblk, total);
   k_scan_add<<<(unsigned)nblk, 1024, 0, st>>>(a, n, tot);
+}
+
+int lbm_sim::build_links() {
+  rplane.assign(nz + 1, 0u);
+  if (has_shell) return LBM_OK;  // never fused
+  const long long nchunk = np / 32, nblk = (nchunk + 1023) / 1024;
+  const unsigned blocks = (unsigned)((np + 255) / 256);
+  // scratch: open links and packed records before each chunk, the scan's block totals, the two totals
+  uint32_t *obase = nullptr;
+  LBM_CUDA_GEO(this, cudaMalloc(&chunk, nchunk * sizeof(uint4)));
+  LBM_CUDA_GEO(this, cudaMalloc(&obase, (2 * nchunk + nblk + 2) * sizeof(uint32_t)));
+  uint32_t *rbase = obase + nchunk, *tot = rbase + nchunk + 1, *total = tot + nblk;
+  std::vector<uint32_t> hr(nchunk + 1);
+  uint32_t nopen = 0;
+  k_geo_lcount<<<blocks, 256, 0, stream>>>(view(), obase, rbase);
+  exclusive_scan(obase, nchunk, tot, total, stream);
+  exclusive_scan(rbase, nchunk, tot, rbase + nchunk, stream);
+  cudaError_t e = cudaMemcpyAsync(&nopen, total, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(hr.data(), rbase, hr.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  if (e == cudaSuccess) {
+    const long long pchunks = (long long)nxp * ny / 32;
+    for (int z = 0; z <= nz; ++z) rplane[z] = hr[z * pchunks];
+    e = cudaMalloc(&ldesc, std::max<long long>(1, nl + nopen) * sizeof(uint16_t));
+  }
+  if (e == cudaSuccess && rplane[nz]) e = cudaMalloc(&rrec, rplane[nz] * sizeof(Rec));
+  if (e == cudaSuccess && rplane[nz]) e = cudaMalloc(&rrnode, rplane[nz] * sizeof(uint32_t));
+  if (e == cudaSuccess) {
+    auto *kern = lattice == LBM_D2Q9 ? k_geo_links<D2Q9> : (lattice == LBM_D3Q19 ? k_geo_links<D3Q19> : k_geo_links<D3Q27>);
+    kern<<<blocks, 256, 0, stream>>>(view(), obase, rbase, flags, chunk, ldesc, rrec, rrnode);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  cudaFree(obase);
+  if (e != cudaSuccess)
+    return lbm_fail(this, e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA,
+                    std::string("links by chunk: ") + cudaGetErrorString(e));
+  return LBM_OK;
 }
 
 extern "C" int lbm_build_geometry(lbm_handle h, const uint8_t *base, const double *base_u,
@@ -1151,6 +1291,9 @@ static int setup_body(lbm_handle h, const lbm_shape *body, const double lo[3], c
   ++h->version;
   h->tiles_bx = h->tiles_by = 0;
   h->drop_graphs();
+  k_move_chunks<<<(unsigned)((mb.rsize + 255) / 256), 256, 0, h->stream>>>(h->view(), mb.ox, mb.oy, mb.oz, mb.rx, mb.ry,
+                                                                           mb.rz, h->chunk);
+  LBM_CUDA_GEO(h, cudaGetLastError());
   // geometry of the first pose for the next step (no refill: the state is set
   // afterwards or was set on the static geometry)
   cudaError_t err = move_geometry(h, 0, 0, h->f[h->cur], h->cur);

@@ -70,14 +70,15 @@ cudaError_t launch_step(int lattice, int dtype, int variant, const View &v, cons
   return dispatch(lattice, dtype, [&]<class L, typename S, typename M>() {
     if (variant == 9 || variant == 10) return launch_split_ls<L, S>(variant, v, fin, fout, l, lb);
     if (variant >= 4 && variant <= 8) return launch_wide_ls<L, S>(variant, v, fin, fout, l);
+    if (v.fused) return launch_bulk_ls<L, S>(variant, v, fin, fout, l, lb);
     return launch_one_ls<L, S>(variant, v, fin, fout, l);
   });
 }
 
-cudaError_t launch_step_batch(int lattice, int dtype, int variant, int phys, const BatchEntry *entries,
+cudaError_t launch_step_batch(int lattice, int dtype, int variant, int kind, int phys, const BatchEntry *entries,
                               const int4 *tiles, int n, int T, int parity, const Launch &l) {
   return dispatch(lattice, dtype, [&]<class L, typename S, typename M>() {
-    return launch_batch_ls<L, S>(variant, phys, entries, tiles, n, T, parity, l);
+    return launch_batch_ls<L, S>(variant, kind, phys, entries, tiles, n, T, parity, l);
   });
 }
 

@@ -774,6 +774,211 @@ __device__ __forceinline__ void lattice_tile(const View &v, const S *__restrict_
   else collide_store_at<L, S, M, PHYS>(v, f, m, fout, n, 0u);
 }
 
+// Rows of a warp's staging array in warp_links: the populations, then drho, rho and u.
+template <class L> constexpr int kStageRows = L::Q + 5;
+
+// The boundary rule of a warp's chunk, one link per lane. The lanes of the chunk's
+// boundary nodes have staged their gathered populations and moments in st
+// ([row][lane]); the links' descriptors say which lane's node and which direction. A
+// lane then evaluates whole links: no node is gathered a second time, no moment is
+// computed twice, and no lane waits for the record with the most links, which is
+// what the record-per-thread boundary tiles cost (in the porous medium 1.94 times
+// the iterations, and a second pass over the boundary nodes' 19 planes). ELIBB-F and
+// -FQ with the bounce-back wall estimate, BGK or TRT; every operation is
+// boundary_rule's, in the units of the stored values, so the values agree bit for bit.
+template <class L, typename S, typename M, int PHYS>
+__device__ __forceinline__ void warp_links(const View &v, const uint4 ck, const M *st, S *__restrict__ fout,
+                                           int n0, int x0, int y, int z) {
+  using X = Ex<M>;
+  constexpr bool FORCE = (PHYS & PH_FORCE) != 0, TRT = (PHYS & PH_TRT) != 0;
+  const int nwall = ck.z & 1023, nlink = nwall + ((ck.z >> 10) & 1023);
+  const bool moving = (ck.z >> 20) != 0;  // some node of the chunk has moving wall links
+  const bool rows_inside = y > 0 && y < v.ny - 1 && (L::D == 2 || (z > 0 && z < v.nz - 1));
+  const Par<M> P(v, Units<S>::kStored);
+#pragma unroll 1
+  for (int k = threadIdx.x & 31; k < nlink; k += 32) {
+    const uint32_t d = __ldg(v.ldesc + (ck.x + k));
+    const bool open = k >= nwall;
+    const uint32_t li = ck.y + k;
+    const M q = open ? M(0.5) : __ldg(static_cast<const M *>(v.lq) + li);
+    const int o = d & 31, i = d >> 5;
+    const float4 dir = __ldg(reinterpret_cast<const float4 *>(v.dirs + i));
+    const M cx = M(dir.x), cy = M(dir.y), cz = M(dir.z);
+    M w;
+    if constexpr (sizeof(M) == 8) w = dweight<L, M>(i); else w = dir.w;
+    const M *col = st + o;
+    const M fi = col[i * 32], fib = col[(L::Q - 1 - i) * 32];
+    const M drho = col[L::Q * 32], rho = col[(L::Q + 1) * 32];
+    const M ux = col[(L::Q + 2) * 32], uy = col[(L::Q + 3) * 32], uz = col[(L::Q + 4) * 32];
+    const M usq = X::fma(uz, uz, X::fma(uy, uy, X::mul(ux, ux)));
+    const M cu = X::fma(cz, uz, X::fma(cy, uy, X::mul(cx, ux)));
+    const M us = X::mul(M(-1.5), usq);
+    const M t_ib = X::fma(X::mul(M(4.5), cu), cu, X::fma(M(3), -cu, us));
+    const M fneq = X::sub(fib, X::mul(w, X::fma(rho, t_ib, drho)));  // f^neq_ibar
+    M val;
+    if (open) {
+      const M t_i = X::fma(X::mul(M(4.5), cu), cu, X::fma(M(3), cu, us));
+      val = X::add(X::mul(w, X::fma(P.rho0, t_i, M(0))), fneq);
+    } else {
+      // post-collision value of ibar (g, with the moving-wall term below), or of i (h)
+      auto post = [&](bool bar) {
+        M r;
+        if constexpr (TRT) {
+          const M ep = X::mul(w, X::fma(rho, X::fma(X::mul(M(4.5), cu), cu, us), drho));
+          const M em = X::mul(X::mul(M(3), w), X::mul(rho, cu));
+          const M fp = X::mul(M(0.5), X::add(fi, fib)), fm = X::mul(M(0.5), X::sub(fi, fib));
+          r = X::fma(P.omega_m, bar ? X::sub(fm, em) : X::sub(em, fm), X::fma(P.omega, X::sub(ep, fp), bar ? fib : fi));
+        } else if (bar) {
+          r = X::fma(P.omega, -fneq, fib);
+        } else {
+          const M t_i = X::fma(X::mul(M(4.5), cu), cu, X::fma(M(3), cu, us));
+          r = X::fma(P.omega, X::sub(X::mul(w, X::fma(rho, t_i, drho)), fi), fi);
+        }
+        if constexpr (FORCE) {
+          const M cF = X::fma(cz, P.F[2], X::fma(cy, P.F[1], X::mul(cx, P.F[0])));
+          const M uF = X::fma(uz, P.F[2], X::fma(uy, P.F[1], X::mul(ux, P.F[0])));
+          const M kp = X::fma(M(-0.5), P.omega, M(1));
+          const M km3 = X::mul(M(3), X::fma(M(-0.5), TRT ? P.omega_m : P.omega, M(1)));
+          const M sp = X::fma(X::mul(M(9), cu), cF, X::mul(M(-3), uF));
+          r = X::fma(w, X::fma(kp, sp, X::mul(km3, bar ? -cF : cF)), r);
+        }
+        return r;
+      };
+      M g = post(true);
+      M e0 = X::mul(w, drho), e1 = e0;  // f^eq_i(rho, u_w) at t+1 and t; walls at rest
+      if (moving && v.luw != nullptr) {
+        const M *a0 = static_cast<const M *>(v.luw) + 3 * li, *a1 = static_cast<const M *>(v.luw1) + 3 * li;
+        const M wx = a0[0], wy = a0[1], wz = a0[2], vx = a1[0], vy = a1[1], vz = a1[2];
+        const M cw = X::fma(cz, wz, X::fma(cy, wy, X::mul(cx, wx)));
+        const M cv = X::fma(cz, vz, X::fma(cy, vy, X::mul(cx, vx)));
+        g = X::add(g, X::mul(X::mul(X::mul(M(6), w), rho), cw));
+        const M u0sq = X::fma(wz, wz, X::fma(wy, wy, X::mul(wx, wx)));
+        const M u1sq = X::fma(vz, vz, X::fma(vy, vy, X::mul(vx, vx)));
+        e1 = X::mul(w, X::fma(rho, X::fma(X::mul(M(4.5), cw), cw, X::fma(M(3), cw, X::mul(M(-1.5), u0sq))), drho));
+        e0 = X::mul(w, X::fma(rho, X::fma(X::mul(M(4.5), cv), cv, X::fma(M(3), cv, X::mul(M(-1.5), u1sq))), drho));
+      }
+      const M f1 = X::fma(X::sub(M(1), P.omega), fneq, e1), f0 = X::add(e0, fneq);
+      const M q2 = X::mul(M(2), q), a = X::sub(q2, M(1)), oma = X::sub(M(1), q2), omq = X::sub(M(1), q);
+      const bool near = q < M(0.5);
+      M num = near ? X::fma(q, g, X::mul(oma, f0)) : X::fma(a, f1, X::mul(omq, g)), den = near ? omq : q;
+      if (v.bc == BC_ELIBB_FQ && !near) {
+        num = X::fma(X::mul(a, X::sub(q, M(1))), post(false), X::fma(X::mul(M(2), a), f1, X::mul(omq, g)));
+        den = X::mul(q2, q);
+      }
+      val = X::div(num, den);
+      if (v.bc == BC_ELIBB_FQ && near && q >= P.qcut) val = X::fma(a, f1, X::fma(oma, f0, g));
+      if (q == M(0.5)) val = g;
+    }
+    // the slot of population i at the upstream node
+    const int x = x0 + o, n = n0 + o;
+    int slot = n + __ldg(&v.dirs[i].off);
+    if (!rows_inside || x == 0 || x == v.nx - 1)
+      slot = i * (int)v.np + n + upstream_offset(v, x, y, z, dcx<L>(i), dcy<L>(i), dcz<L>(i));
+    ST_POP(v, fout, &fout[slot], Units<S>::template store<M>(val));
+  }
+}
+
+// ---------------------------------------------------------------- bulk tiles
+// One row of a bulk tile: this warp's chunk of row (y, z). The step's instruction
+// count, not memory, bounds FP16 storage and the porous medium (74-77 % of the issue
+// slots taken; 565 and 960 instructions a warp through the tile table and the flags,
+// 434 and 760 here), so the chunk's kind is decided when the geometry is set:
+//  - CK_PLAIN chunks (three quarters of a 256-node duct row) load no flags, test
+//    nothing and store whole sectors: 19 loads, the relaxation, 19 stores;
+//  - CK_IDLE chunks leave at once;
+//  - the others look at the flags. The x wrap costs them no second gather: the
+//    sources of c_x = +1 and -1 are addressed through an index of their own that
+//    carries the wrap of the lane at the row's end. Only rows at the y and z edges,
+//    and sheared row ends, gather through the wrap table.
+// Every plane has its own pointer (Planes), a constant operand, so that an address is
+// one multiply-add. Walking the planes instead, by 64-bit or by 32-bit steps, takes 10 %
+// more instructions and was slower (porous FP16, 192^3: 206 and 204 against 187 us).
+// A non-fluid node whose 32-byte sector holds a fluid node stores the relaxation of
+// zeros into the planes that take no written-ahead value, as in lattice_tile. The
+// nodes' arithmetic is lattice_tile's, operation for operation.
+template <class L, typename S, typename M, int PHYS, bool LINKS>
+__device__ __forceinline__ void bulk_row(const View &v, const Planes &p, M *st, int x, int y, int z) {
+  using U = Units<S>;
+  const int n = (z * v.ny + y) * v.nxp + x;
+  const uint4 ck = __ldg(v.chunk + (n >> 5));
+  if (ck.w & CK_IDLE) return;
+  const S *fin = static_cast<const S *>(p.fin);
+  S *fout = static_cast<S *>(p.fout);
+  const unsigned un = (unsigned)n;
+  const bool links = LINKS && (ck.w & CK_LINKS);
+  M f[L::Q];
+  if ((ck.w & CK_PLAIN) && !links) {
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) f[i] = U::template load<M>(LD_POP(v, fin, static_cast<const S *>(p.src[i]) + un));
+    const Macro<L, M> m = moments<L, M, U::kStored>(v, f);
+    relax<L, M, PHYS, U::kStored>(v, f, m, [&](int i, M val) {
+      ST_POP(v, fout, static_cast<S *>(p.dst[i]) + un, U::template store<M>(val));
+    });
+    return;
+  }
+  const uint8_t fl = v.flags[n];
+  const uint32_t fbal = __ballot_sync(0xffffffffu, (fl & 3) == K_FLUID);
+  const bool here = (fl & 3) == K_FLUID;
+  const bool fill = fills_sector<S>(fl, fbal, 1);     // a non-fluid node completing a sector
+  const bool masked = __any_sync(0xffffffffu, fill);  // the warp's stores need the per-plane masks
+  const bool rows_inside = y > 0 && y < v.ny - 1 && (L::D == 2 || (z > 0 && z < v.nz - 1));
+  uint32_t skip = 0;
+  if (here) {
+    if (rows_inside && (v.xshift == 0 || (x > 0 && x < v.nx - 1))) {
+      const unsigned up = un + (x == 0 ? v.nx : 0), dn = un - (x == v.nx - 1 ? v.nx : 0);
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i)
+        f[i] = U::template load<M>(
+            LD_POP(v, fin, static_cast<const S *>(p.src[i]) + (L::cx(i) > 0 ? up : (L::cx(i) < 0 ? dn : un))));
+    } else {
+      Nbr nb;
+      nb.init(v, x, y, z);
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i)
+        f[i] = U::template load<M>(
+            LD_POP(v, fin, fin + (n + (i * (int)v.np + nb.at(-L::cx(i), -L::cy(i), -L::cz(i))))));
+    }
+  } else {
+    if (fill) skip = v.amask[n];
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) f[i] = M(0);
+  }
+  if (links) {
+    // the links' data, asked for while the gather is in flight
+    const int lane = threadIdx.x & 31, nwall = ck.z & 1023, nlink = nwall + ((ck.z >> 10) & 1023);
+    if (nwall > 0 && lane * 32 < nwall + 31)
+      prefetch_l1(static_cast<const M *>(v.lq) + ck.y + min(lane * 32, nwall - 1));
+    if (lane * 64 < nlink + 63) prefetch_l1(v.ldesc + ck.x + min(lane * 64, nlink - 1));
+  }
+  if (here || fill) {
+    const Macro<L, M> m = moments<L, M, U::kStored>(v, f);
+    if (LINKS && (fl & F_LINKS)) {
+      M *col = st + (threadIdx.x & 31);
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i) col[i * 32] = f[i];
+      col[L::Q * 32] = m.drho;
+      col[(L::Q + 1) * 32] = m.rho;
+      col[(L::Q + 2) * 32] = m.ux;
+      col[(L::Q + 3) * 32] = m.uy;
+      col[(L::Q + 4) * 32] = m.uz;
+    }
+    if (masked)
+      relax<L, M, PHYS, U::kStored>(v, f, m, [&](int i, M val) {
+        if (!((skip >> i) & 1u)) ST_POP(v, fout, static_cast<S *>(p.dst[i]) + un, U::template store<M>(val));
+      });
+    else
+      relax<L, M, PHYS, U::kStored>(v, f, m, [&](int i, M val) {
+        ST_POP(v, fout, static_cast<S *>(p.dst[i]) + un, U::template store<M>(val));
+      });
+  }
+  if (links) {
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    warp_links<L, S, M, PHYS>(v, ck, st, fout, n - lane, x - lane, y, z);
+    __syncwarp();  // the staging array is free for the warp's next row
+  }
+}
+
 // ---------------------------------------------------------------- two nodes per thread
 // Lattice tile {z, t} with bx threads covering 2 bx nodes of a row: thread tx owns
 // the aligned pair (x, x+1), x = x0 + 2 tx. One vector load per plane fetches the
@@ -939,12 +1144,20 @@ __device__ __forceinline__ void boundary_tile(const View &v, const S *__restrict
   const int tpb = (int)(blockDim.x * blockDim.y);
   const int count = dyn ? min(tpb, *v.dyn_count - tile.y) : -1 - tile.x;
   if (t >= count) return;
-  const RecSet rs = dyn ? v.dyn : v.stat();
+  const RecSet rs = dyn ? v.dyn : RecSet{v.trec, v.trnode, v.lq, v.luw, v.luw1, v.ltag};
   const int rid = tile.y + t;
   const Rec r = rs.rec[rid];
   const int n = (int)rs.rnode[rid];
   const int3 c = node_coords(v, n);
-  boundary_node<L, S, M>(v, rs, r, fin, fout, n, c.x, c.y, c.z, stage + t, stage_threads<L, M>());
+  boundary_node<L, S, M>(v, rs, r, fin, fout, n, c.x, c.y, c.z, stage + t, tpb);
+}
+
+// Dynamic shared memory of the step kernels: sized by the launch (step_smem) for
+// the block's own threads, so that small blocks leave the rest to L1 and to other blocks.
+template <typename M>
+__device__ __forceinline__ M *step_stage() {
+  extern __shared__ __align__(16) unsigned char step_smem_raw[];
+  return reinterpret_cast<M *>(step_smem_raw);
 }
 
 // Block b takes table entries b*T .. b*T+T-1 (T = v.tpb_tiles <= 4), whose
@@ -953,7 +1166,7 @@ __device__ __forceinline__ void boundary_tile(const View &v, const S *__restrict
 template <class L, typename S, typename M, int MINB, int PHYS, bool PAIR = false, int MAXT = 256>
 __global__ void __launch_bounds__(MAXT, MINB) k_step(const __grid_constant__ View v, const S *__restrict__ fin,
                                                      S *__restrict__ fout) {
-  __shared__ M stage[L::Q * stage_threads<L, M>()];  // boundary tiles: populations, [direction][thread]
+  M *stage = step_stage<M>();  // boundary tiles: populations, [direction][thread]
   const int T = v.tpb_tiles;
   const int first = blockIdx.x * T;
   int2 tl[4];
@@ -998,8 +1211,22 @@ __global__ void __launch_bounds__(256, MINB) k_lattice(const __grid_constant__ V
 template <class L, typename S, typename M>
 __global__ void __launch_bounds__(256, 4) k_boundary(const __grid_constant__ View v, const S *__restrict__ fin,
                                                      S *__restrict__ fout) {
-  __shared__ M stage[L::Q * stage_threads<L, M>()];  // populations, [direction][thread]
-  boundary_tile<L, S, M>(v, fin, fout, v.btiles[blockIdx.x], stage);
+  boundary_tile<L, S, M>(v, fin, fout, v.btiles[blockIdx.x], step_stage<M>());  // populations, [direction][thread]
+}
+
+// ---------------------------------------------------------------- bulk step
+// The one-node launches under View::fused: the grid is the lattice itself (blocks of bx
+// by by nodes, T of them one above the other per block), no tile table. The records of
+// the chunks without F_LINKS, and a moving body's, go to k_boundary beside it, as in
+// the split step.
+template <class L, typename S, typename M, int MINB, int PHYS>
+__global__ void __launch_bounds__(256, MINB) k_bulk(const __grid_constant__ View v, const __grid_constant__ Planes p) {
+  M *st = step_stage<M>() + ((threadIdx.y * blockDim.x + threadIdx.x) >> 5) * (kStageRows<L> * 32);
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, T = v.tpb_tiles;
+  int y = blockIdx.y * T * blockDim.y + threadIdx.y;
+#pragma unroll 1
+  for (int k = 0; k < T; ++k, y += blockDim.y)
+    if (y < v.ny) bulk_row<L, S, M, PHYS, true>(v, p, st, x, y, blockIdx.z);
 }
 
 // ---------------------------------------------------------------- TMA-staged step
@@ -1226,52 +1453,98 @@ __global__ void __launch_bounds__(256, 2) k_step_tma(const __grid_constant__ Vie
 }
 
 // ---------------------------------------------------------------- batched step
-// Many independent simulations advance in one launch. Entry k holds the view
-// and the two population buffers of simulation k. The tile table lists
-// {sim, z, t, 0} lattice tiles and {sim, -1, first, count} boundary tiles, one
-// simulation after another, each plane-interleaved as in k_step. parity picks
-// which buffer of each entry is read in this step. A block copies the entry of
-// its tile into shared memory. The table is grouped by physics class (body
-// force, collision operator), and one launch covers one class, compiled for it
-// (PHYS) as k_step is. The per-node code is the same as k_step's, so a batched
-// simulation gives exactly the results it gives when stepped alone.
+// Many independent simulations advance in one launch per kernel. Entry k holds the
+// view and the two population buffers of simulation k; parity picks which buffer of
+// each entry is read in this step. A block copies the entry of its tile into shared
+// memory. The per-node code is the single simulation's, so a batched simulation gives
+// exactly the results it gives when stepped alone. The tables are grouped by physics
+// class (body force, collision operator), and one launch covers one class, compiled
+// for it (PHYS) as the single simulation's kernels are:
+//  - k_bulk_batch takes the bulk tiles {sim, z, x tile, y tile} of the simulations
+//    under View::fused, and k_boundary_batch their boundary tiles {sim, -1, first,
+//    count}, side by side as in the bulk step;
+//  - k_step_batch takes the other simulations' lattice tiles {sim, z, t, 0} and
+//    boundary tiles, one simulation after another, each plane-interleaved as in k_step.
 struct alignas(16) BatchEntry {
   View v;
   const void *f0;  // read on even batch steps
   void *f1;        // read on odd batch steps
 };
 
+// The block's copy of an entry: made when a tile belongs to another simulation than
+// the one held (uniform across the block). The first warp copies it in 16-byte pieces.
+__device__ __forceinline__ bool hold_entry(BatchEntry &se, const BatchEntry *__restrict__ entries, int sim, int &held) {
+  if (sim == held) return false;
+  __syncthreads();  // the previous tile is done with se
+  constexpr int kPieces = (int)(sizeof(BatchEntry) / 16);
+  const int4 *src = reinterpret_cast<const int4 *>(entries + sim);
+  int4 *dst = reinterpret_cast<int4 *>(&se);
+  const int t = threadIdx.y * blockDim.x + threadIdx.x;
+  if (t < 32)
+    for (int k = t; k < kPieces; k += 32) dst[k] = __ldg(src + k);
+  __syncthreads();
+  held = sim;
+  return true;
+}
+
 template <class L, typename S, typename M, int MINB, int PHYS>
 __global__ void __launch_bounds__(256, MINB) k_step_batch(const BatchEntry *__restrict__ entries,
                                                           const int4 *__restrict__ tiles, int ntiles,
                                                           int T, int parity) {
-  __shared__ M stage[L::Q * stage_threads<L, M>()];
+  M *stage = step_stage<M>();
   __shared__ BatchEntry se;
-  const int t = threadIdx.y * blockDim.x + threadIdx.x;
   int held = -1;  // the entry in se; a block's tiles mostly belong to one simulation
   for (int k = 0; k < T; ++k) {
     const int idx = blockIdx.x * T + k;
     if (idx >= ntiles) break;  // uniform across the block
     const int4 tile = tiles[idx];
-    if (tile.x != held) {  // uniform across the block
-      __syncthreads();  // the previous tile is done with se
-      {  // the first warp copies the entry in 16-byte pieces
-        constexpr int kPieces = (int)(sizeof(BatchEntry) / 16);
-        const int4 *src = reinterpret_cast<const int4 *>(entries + tile.x);
-        int4 *dst = reinterpret_cast<int4 *>(&se);
-        if (t < 32)
-          for (int k = t; k < kPieces; k += 32) dst[k] = __ldg(src + k);
-      }
-      __syncthreads();
-      held = tile.x;
-    }
+    hold_entry(se, entries, tile.x, held);
     const S *fin = static_cast<const S *>(parity ? se.f1 : se.f0);
     S *fout = static_cast<S *>(parity ? const_cast<void *>(se.f0) : se.f1);
-    // each simulation takes the same compiled path as when it steps alone: the
-    // launch covers the simulations of one physics class (PHYS) only
     if (tile.y < 0) boundary_tile<L, S, M>(se.v, fin, fout, make_int2(-1 - tile.w, tile.z), stage);
     else lattice_tile<L, S, M, PHYS>(se.v, fin, fout, make_int2(tile.y, tile.z));
   }
+}
+
+template <class L, typename S, typename M, int MINB, int PHYS>
+__global__ void __launch_bounds__(256, MINB) k_bulk_batch(const BatchEntry *__restrict__ entries,
+                                                          const int4 *__restrict__ tiles, int ntiles,
+                                                          int T, int parity) {
+  __shared__ BatchEntry se;
+  __shared__ Planes pl;
+  const int t = threadIdx.y * blockDim.x + threadIdx.x;
+  M *st = step_stage<M>() + (t >> 5) * (kStageRows<L> * 32);
+  int held = -1;
+  for (int k = 0; k < T; ++k) {
+    const int idx = blockIdx.x * T + k;
+    if (idx >= ntiles) break;  // uniform across the block
+    const int4 tile = tiles[idx];
+    if (hold_entry(se, entries, tile.x, held)) {
+      if (t < L::Q) {
+        pl.src[t] = static_cast<const S *>(parity ? se.f1 : se.f0) + se.v.loff[t];
+        pl.dst[t] = static_cast<S *>(parity ? const_cast<void *>(se.f0) : se.f1) + se.v.soff[t];
+      }
+      if (t == 0) {
+        pl.fin = parity ? se.f1 : se.f0;
+        pl.fout = parity ? const_cast<void *>(se.f0) : se.f1;
+      }
+      __syncthreads();
+    }
+    const int y = tile.w * blockDim.y + threadIdx.y;
+    if (y < se.v.ny) bulk_row<L, S, M, PHYS, true>(se.v, pl, st, tile.z * blockDim.x + threadIdx.x, y, tile.y);
+  }
+}
+
+template <class L, typename S, typename M>
+__global__ void __launch_bounds__(256, 4) k_boundary_batch(const BatchEntry *__restrict__ entries,
+                                                           const int4 *__restrict__ tiles, int parity) {
+  __shared__ BatchEntry se;
+  int held = -1;
+  const int4 tile = tiles[blockIdx.x];
+  hold_entry(se, entries, tile.x, held);
+  boundary_tile<L, S, M>(se.v, static_cast<const S *>(parity ? se.f1 : se.f0),
+                         static_cast<S *>(parity ? const_cast<void *>(se.f0) : se.f1),
+                         make_int2(-1 - tile.w, tile.z), step_stage<M>());
 }
 
 // ---------------------------------------------------------------- state set-up and read-out

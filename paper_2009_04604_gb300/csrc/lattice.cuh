@@ -145,7 +145,9 @@ template <> __device__ __forceinline__ __nv_bfloat16 to_store<__nv_bfloat16, flo
 // Bit 4 marks the nodes of a moving body's region: the lattice tiles never store
 // into a non-fluid node's slots there (values are written ahead into them, and
 // which ones changes every step).
-enum : uint8_t { K_FLUID = 0, K_SOLID = 1, K_OPEN = 2, K_PAD = 3, F_BOUNDARY = 4, F_SHELL = 8, F_KEEP = 16 };
+// Bit 5 marks the boundary nodes of the chunks whose links the lattice tiles evaluate
+// under View::fused (lbm_sim::build_links); not part of the geometry's hash.
+enum : uint8_t { K_FLUID = 0, K_SOLID = 1, K_OPEN = 2, K_PAD = 3, F_BOUNDARY = 4, F_SHELL = 8, F_KEEP = 16, F_LINKS = 32 };
 // Flag bits a lattice tile tests: it relaxes the node only when they are all zero.
 constexpr uint8_t K_LATTICE_MASK = 3 | F_SHELL;
 // Force tag of the links on the inner side of a thin shell: no force is counted there.
@@ -159,6 +161,29 @@ struct Rec {
   uint32_t ffok;  // bit i: the second node along the link, n + c_i, is fluid and on this side (BFL)
   uint32_t link0; // index of the first wall link of this node in the link arrays
   uint32_t shell; // bit i: link i crosses a thin shell to the fluid node n - c_i (also in cut)
+};
+
+// Link descriptor: owner lane (bits 0-4) and direction (5-9).
+__host__ __device__ constexpr uint16_t link_desc(int lane, int i) { return (uint16_t)(lane | i << 5); }
+
+// A direction for a link chosen at run time: one 16-byte load gives its velocity and
+// weight, another the offset of its slot at the upstream node (View::loff).
+struct alignas(16) LinkDir {
+  float cx, cy, cz, w;
+  int off, pad[3];
+};
+
+// Chunk bits: every node fluid, off the lattice's edges and outside a moving body's
+// region; no fluid node; links to evaluate (F_LINKS nodes).
+enum : uint32_t { CK_PLAIN = 1, CK_IDLE = 2, CK_LINKS = 4 };
+
+// Where the bulk tiles find node n's populations: src[i] + n, the source of
+// population i without a wrap (fin + loff[i]), and dst[i] + n (fout + soff[i]).
+struct Planes {
+  const void *src[27];
+  void *dst[27];
+  const void *fin;
+  void *fout;
 };
 
 // One set of boundary records and their per-link data (math type).
@@ -206,6 +231,16 @@ struct View {
   int soff[27], loff[27];
   int ntiles, tpb_tiles;     // table length; consecutive table entries per block
   const int2 *btiles;        // split step (variants 9, 10): the boundary entries, apart from v.tiles
+  // 32-node chunks for the bulk tiles (bulk_row): {first link descriptor, first wall link,
+  // wall links | open links << 10 | moving << 20, CK_* bits}, and a 16-bit descriptor per
+  // link, in chunk order, the wall links (in the order of lq) before the open ones
+  int fused;                 // 1: the step runs bulk tiles, which write the values of the F_LINKS nodes' links ahead
+  const uint4 *chunk;
+  const uint16_t *ldesc;
+  const LinkDir *dirs;       // [Q]
+  // the static records of the boundary tiles: all, or those without F_LINKS under fused
+  const Rec *trec;
+  const uint32_t *trnode;
   // moving body: records of the nodes of its region, rebuilt every step
   RecSet dyn;
   const int *dyn_count;      // device: number of records in dyn (null: no moving body)

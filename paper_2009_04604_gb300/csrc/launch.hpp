@@ -32,10 +32,12 @@ cudaError_t prepare_step_tma(int lattice, int dtype, int phys, int bx, int by, l
 // variant.
 cudaError_t launch_step(int lattice, int dtype, int variant, const View &v, const void *fin,
                         void *fout, const Launch &l, const Launch *lb = nullptr);
-// One launch of the batched step: the n tiles of one physics class (PH_FORCE | PH_TRT
-// bits), T consecutive ones per block; parity picks which buffer of each entry is read.
+// One launch of the batched step: n tiles of one kind and physics class (PH_FORCE |
+// PH_TRT bits; boundary tiles have none), T consecutive ones per block; parity picks
+// which buffer of each entry is read.
 struct BatchEntry;
-cudaError_t launch_step_batch(int lattice, int dtype, int variant, int phys, const BatchEntry *entries,
+enum { kBatchBulk = 0, kBatchBoundary = 1, kBatchStep = 2 };
+cudaError_t launch_step_batch(int lattice, int dtype, int variant, int kind, int phys, const BatchEntry *entries,
                               const int4 *tiles, int n, int T, int parity, const Launch &l);
 cudaError_t launch_init(int lattice, int dtype, const View &v, void *fout, double rho, double ux,
                         double uy, double uz, const Launch &l);

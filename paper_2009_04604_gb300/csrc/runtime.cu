@@ -121,6 +121,21 @@ extern "C" int lbm_create(int lattice, const int dims[3], double tau, int dtype,
     lbm_destroy(h);
     return lbm_fail(nullptr, e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA, msg);
   }
+  {
+    const View v = h->view();
+    LinkDir d[27] = {};
+    for (int i = 0; i < h->Q; ++i) {
+      int c[3];
+      h->lattice_c(i, c[0], c[1], c[2]);
+      d[i] = LinkDir{(float)c[0], (float)c[1], (float)c[2], (float)h->lattice_w(i), v.loff[i], {0, 0, 0}};
+    }
+    e = cudaMalloc(&h->dirs, sizeof(d));
+    if (e == cudaSuccess) e = cudaMemcpy(h->dirs, d, sizeof(d), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      lbm_destroy(h);
+      return lbm_fail(nullptr, e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA, cudaGetErrorString(e));
+    }
+  }
   h->tune_default();
   *out = h;
   return LBM_OK;
@@ -128,6 +143,8 @@ extern "C" int lbm_create(int lattice, const int dims[3], double tau, int dtype,
 
 void lbm_sim::free_geometry() {
   cudaFree(rec); cudaFree(rnode); cudaFree(lq); cudaFree(luw); cudaFree(luw1); cudaFree(ltag);
+  cudaFree(chunk); cudaFree(ldesc); cudaFree(rrec); cudaFree(rrnode);
+  chunk = nullptr; ldesc = nullptr; rrec = nullptr; rrnode = nullptr;
   rec = nullptr; rnode = nullptr; lq = nullptr; luw = nullptr; luw1 = nullptr; ltag = nullptr;
   nb = nl = 0;
   has_uw = 0;
@@ -154,12 +171,14 @@ static unsigned long long fnv_words(unsigned long long h, const void *p, size_t 
 }
 
 // After a static geometry is in place: the written-ahead masks of the non-fluid
-// nodes (View::amask) and the geometry's hash (for lbm_save / lbm_load).
+// nodes (View::amask), the links by chunk (View::chunk) and the geometry's hash (for
+// lbm_save / lbm_load).
 int lbm_sim::finish_geometry() {
   LBM_CUDA(this, launch_amask(lattice, view(), amask, stream));
   HostGeometry g;
   int rc = download(g);
   if (rc) return rc;
+  if (!launch_set) tune_default();  // thin shells step through the tile table
   unsigned long long h = 0xcbf29ce484222325ULL;
   const long long dims[5] = {lattice, nx, ny, nz, dtype};
   h = fnv_words(h, dims, sizeof(dims));
@@ -171,7 +190,7 @@ int lbm_sim::finish_geometry() {
   h = fnv_words(h, g.luw.data(), g.luw.size());
   h = fnv_words(h, g.luw1.data(), g.luw1.size());
   geom_hash = h;
-  return LBM_OK;
+  return build_links();  // after the hash: it marks nodes in the flags
 }
 
 void lbm_sim::drop_graphs() {
@@ -187,7 +206,7 @@ extern "C" int lbm_destroy(lbm_handle h) {
   cudaFree(h->f[0]); cudaFree(h->f[1]); cudaFree(h->flags); cudaFree(h->cbase);
   cudaFree(h->dres); cudaFree(h->scratch); cudaFree(h->tiles); cudaFree(h->err_dev); cudaFree(h->dbg_dev);
   cudaFree(h->btiles);
-  cudaFree(h->amask); cudaFree(h->stage_f);
+  cudaFree(h->amask); cudaFree(h->stage_f); cudaFree(h->dirs);
   h->free_moving_body();
   if (h->aux) { cudaStreamSynchronize(h->aux); cudaStreamDestroy(h->aux); }
   if (h->ev_fork) cudaEventDestroy(h->ev_fork);
@@ -247,7 +266,7 @@ extern "C" int lbm_set_options(lbm_handle h, int bc, double rho0, const double f
     if (e != cudaSuccess) { h->bc = old_bc; return lbm_fail(h, LBM_ERR_CUDA, cudaGetErrorString(e)); }
   }
   h->bc = bc;
-  if (bc == LBM_BC_BFL && h->npt() == 2) { h->variant = 0; h->tune_default(); }  // pairs have no BFL path
+  if (bc == LBM_BC_BFL && h->npt() == 2) { h->variant = 0; h->wide_shape(); }  // pairs have no BFL path
   h->rho0 = rho0;
   h->has_force = 0;
   for (int a = 0; a < 3; ++a) {
@@ -256,6 +275,7 @@ extern "C" int lbm_set_options(lbm_handle h, int bc, double rho0, const double f
   }
   if (h->lattice == LBM_D2Q9) { h->F[2] = 0.0; }
   h->xshift = xshift;
+  if (!h->launch_set) h->tune_default();
   h->drop_graphs();
   h->tiles_var = -1;  // the TMA-staged step is prepared per force path
   ++h->version;
@@ -267,6 +287,7 @@ extern "C" int lbm_set_wall_neq(lbm_handle h, int mode) {
   if (mode != LBM_NEQ_BOUNCE_BACK && mode != LBM_NEQ_REGULARIZED)
     return lbm_fail(h, LBM_ERR_ARG, "unknown wall non-equilibrium estimate");
   h->wall_neq = mode;
+  if (!h->launch_set) h->tune_default();
   h->drop_graphs();
   ++h->version;
   return LBM_OK;
@@ -279,6 +300,7 @@ extern "C" int lbm_set_collision(lbm_handle h, int model, double magic) {
     return lbm_fail(h, LBM_ERR_ARG, "the TRT magic parameter must be positive");
   h->collision = model;
   if (model == LBM_COLL_TRT) h->magic = magic;
+  if (!h->launch_set) h->tune_default();
   h->drop_graphs();
   h->tiles_var = -1;  // the TMA-staged step is prepared per collision
   ++h->version;
@@ -331,6 +353,12 @@ View lbm_sim::view() const {
   }
   v.ntiles = (int)ntiles; v.tpb_tiles = tiles_per_block;
   v.btiles = btiles;
+  v.fused = fused() ? 1 : 0;
+  v.trec = v.fused ? rrec : rec;
+  v.trnode = v.fused ? rrnode : rnode;
+  v.chunk = chunk;
+  v.ldesc = ldesc;
+  v.dirs = dirs;
   if (mb.on) {
     v.dyn = RecSet{mb.rec[cur], mb.rnode[cur], mb.lq[cur], mb.luw[cur], mb.luw1[cur], mb.ltag[cur]};
     v.dyn_count = mb.count[cur];
@@ -351,8 +379,9 @@ Launch lbm_sim::shape(int bx, int by) const {
   return l;
 }
 
-void lbm_sim::tune_default() {
-  // widest power-of-two multiple of 32 (<= 128) that divides the padded row
+// The block shape of a launch whose variant the library had to change (BFL has no node
+// pairs): the widest power-of-two multiple of 32 (<= 128) that divides the padded row.
+void lbm_sim::wide_shape() {
   int bx = 32;
   while (bx < 128 && nxp % (bx * 2) == 0) bx *= 2;
   step_bx = bx;
@@ -360,11 +389,46 @@ void lbm_sim::tune_default() {
   step_by = std::max(1, threads / bx);
 }
 
+// The launch until lbm_set_launch or lbm_autotune chooses one. A warp of a one-node
+// kernel covers 32 nodes of a row; what matters is that the warps spread over the SMs
+// and that a small lattice is not stepped by a few blocks one tile after another:
+//  - FP64: the pipe issues 2 lanes per clock and SM, so a step takes as long as the SM
+//    with the most warps. One warp per block up to 16 warps an SM (64 x 64 D2Q9:
+//    35 us a step in 4 blocks of 64 x 4 nodes x 4 tiles, 7.8 in 128 blocks;
+//    64 x 32 x 32 D3Q19: 129 and 50), then two.
+//  - FP32 and below: blocks of 32 x 4 nodes, the best or within 2 % of it at every size
+//    and lattice timed. One tile per block, and two once there are at least four
+//    blocks for every resident one (256 x 128 x 128 duct, FP16: 82.0 us with one, 80.7
+//    with two; 128 x 96 x 80, FP32: 29.3 and 30.1).
+//  - Register budget: 48 for the bulk kernels of D2Q9 and D3Q19 (D3Q19 duct, FP16: 80.7
+//    us, 83.6 at 64, 84.3 at 40), 64 where they would spill more than a few words (D3Q27,
+//    and a body force under TRT) and for the kernels of the tile table.
+void lbm_sim::tune_default() {
+  const long long warps = np / 32;
+  step_bx = 32;
+  tiles_per_block = 1;
+  if (dtype == LBM_F64) {
+    variant = 0;
+    step_by = warps <= 16 * 152 ? 1 : 2;
+    return;
+  }
+  step_by = 4;
+  variant = 11;
+  const bool heavy = lattice == LBM_D3Q27 || (has_force && collision == LBM_COLL_TRT);
+  if (!fused() || heavy) variant = 3;
+  if (warps >= 4LL * 4 * 152 * 10) tiles_per_block = 2;
+}
+
 Launch lbm_sim::step_shape() const {
   Launch l;
   l.block = dim3(step_bx, step_by, 1);
   l.grid = dim3((unsigned)((ntiles + tiles_per_block - 1) / tiles_per_block), 1, 1);
   l.stream = stream;
+  l.smem = step_smem(step_bx * step_by, !split() && (nb > 0 || mb.on), fused());
+  if (fused()) {
+    const int rows = step_by * tiles_per_block;
+    l.grid = dim3(nxp / step_bx, (ny + rows - 1) / rows, nz);
+  }
   if (variant == 4) {
     l.grid = dim3((unsigned)tma_blocks, 1, 1);
     l.smem = tma_smem;
@@ -374,24 +438,28 @@ Launch lbm_sim::step_shape() const {
 
 // Tile table of the step kernel for the current geometry and launch shape: for
 // each plane z, its lattice tiles {z, t} (t = tile in the plane), then its
-// boundary tiles {-1 - count, first record}. The split step keeps the boundary
-// tiles in a table of their own (btiles), in the same order.
+// boundary tiles {-1 - count, first record}. The split step and the bulk step keep
+// the boundary tiles in a table of their own (btiles), in the same order; the bulk
+// step needs no lattice entries.
 int lbm_sim::ensure_tiles() {
-  if (tiles && tiles_bx == step_bx && tiles_by == step_by && tiles_var == variant) return LBM_OK;
+  if (tiles && tiles_bx == step_bx && tiles_by == step_by && tiles_var == variant && tiles_fused == fused())
+    return LBM_OK;
   const int tpb = step_bx * step_by;
   const int gx = nxp / (step_bx * npt()), gy = (ny + step_by - 1) / step_by;
-  std::vector<uint32_t> hc(np / 32 + 1, 0u);
-  if (nb > 0)
+  // records before each plane's first: all of them, or the ones left to the boundary tiles (fused)
+  const long long pchunks = (long long)nxp * ny / 32;
+  std::vector<uint32_t> hc(fused() || nb == 0 ? 0 : np / 32 + 1, 0u);
+  if (!hc.empty())
     LBM_CUDA(this, cudaMemcpyAsync(hc.data(), cbase, hc.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
   LBM_CUDA(this, cudaStreamSynchronize(stream));
   std::vector<int2> t, bt;
   std::vector<int2> &bdst = split() ? bt : t;
-  t.reserve((size_t)nz * gx * gy + nb / tpb + nz + 1);
-  const long long pchunks = (long long)nxp * ny / 32;
+  if (!fused()) t.reserve((size_t)nz * gx * gy + nb / tpb + nz + 1);
   for (int z = 0; z < nz; ++z) {
-    for (int k = 0; k < gx * gy; ++k) t.push_back(make_int2(z, k));
+    if (!fused())
+      for (int k = 0; k < gx * gy; ++k) t.push_back(make_int2(z, k));
     if (nb == 0) continue;
-    const long long r0 = hc[z * pchunks], r1 = hc[(z + 1) * pchunks];
+    const long long r0 = fused() ? rplane[z] : hc[z * pchunks], r1 = fused() ? rplane[z + 1] : hc[(z + 1) * pchunks];
     for (long long r = r0; r < r1; r += tpb)
       bdst.push_back(make_int2(-1 - (int)std::min<long long>(tpb, r1 - r), (int)r));
   }
@@ -403,8 +471,9 @@ int lbm_sim::ensure_tiles() {
   btiles = nullptr;
   ntiles = (long long)t.size();
   nbtiles = (long long)bt.size();
-  LBM_CUDA(this, cudaMalloc(&tiles, ntiles * sizeof(int2)));
-  LBM_CUDA(this, cudaMemcpyAsync(tiles, t.data(), ntiles * sizeof(int2), cudaMemcpyHostToDevice, stream));
+  LBM_CUDA(this, cudaMalloc(&tiles, std::max<long long>(1, ntiles) * sizeof(int2)));
+  if (ntiles)
+    LBM_CUDA(this, cudaMemcpyAsync(tiles, t.data(), ntiles * sizeof(int2), cudaMemcpyHostToDevice, stream));
   if (nbtiles > 0) {
     LBM_CUDA(this, cudaMalloc(&btiles, nbtiles * sizeof(int2)));
     LBM_CUDA(this, cudaMemcpyAsync(btiles, bt.data(), nbtiles * sizeof(int2), cudaMemcpyHostToDevice, stream));
@@ -420,6 +489,7 @@ int lbm_sim::ensure_tiles() {
   tiles_bx = step_bx;
   tiles_by = step_by;
   tiles_var = variant;
+  tiles_fused = fused();
   if (variant == 4) {
     const int phys = (has_force ? PH_FORCE : 0) | (collision == LBM_COLL_TRT ? PH_TRT : 0);
     cudaError_t e = prepare_step_tma(lattice, dtype, phys, step_bx, step_by, ntiles, &tma_blocks, &tma_smem);
@@ -588,6 +658,7 @@ int lbm_sim::launch_steps(int n) {
       Launch lb;
       lb.grid = dim3((unsigned)nbtiles, 1, 1);
       lb.block = dim3(step_bx, step_by, 1);
+      lb.smem = step_smem(step_bx * step_by, true, false);
       lb.stream = aux;
       e = cudaEventRecord(ev_fork, stream);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(aux, ev_fork, 0);
@@ -755,6 +826,7 @@ extern "C" int lbm_set_launch(lbm_handle h, int bx, int by, int variant, int til
   h->step_by = by;
   h->variant = variant;
   h->tiles_per_block = tiles;
+  h->launch_set = true;
   h->drop_graphs();
   return LBM_OK;
 }
@@ -788,6 +860,7 @@ extern "C" int lbm_autotune(lbm_handle h, int steps, int *bx, int *by, int *vari
       for (int var = 0; var < nvar && rc == LBM_OK; ++var)
         for (int k = 0; k < 3 && rc == LBM_OK; ++k) {
           if (var == 4 && k > 0) continue;  // the persistent kernel ignores tiles per block
+          if (var == 1 || var == 2 || var == 6) continue;  // the kernels of 0, 0 and 5
           if (!valid_launch(h, bxx, threads / bxx, var, tile_opts[k])) continue;
           h->step_bx = bxx;
           h->step_by = threads / bxx;
@@ -816,6 +889,7 @@ extern "C" int lbm_autotune(lbm_handle h, int steps, int *bx, int *by, int *vari
   h->step_by = best[1];
   h->variant = best[2];
   h->tiles_per_block = best[3];
+  h->launch_set = true;
   h->drop_graphs();
   if (bx) *bx = best[0];
   if (by) *by = best[1];

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <string>
+#include <vector>
 
 #include "lattice.cuh"
 #include "launch.hpp"
@@ -72,6 +73,12 @@ struct lbm_sim {
   uint32_t *rnode = nullptr;
   void *lq = nullptr, *luw = nullptr, *luw1 = nullptr;
   uint8_t *ltag = nullptr;
+  lbm::LinkDir *dirs = nullptr; // [Q] (View::dirs)
+  uint4 *chunk = nullptr;       // the 32-node chunks and their links (View::chunk, View::ldesc)
+  uint16_t *ldesc = nullptr;
+  lbm::Rec *rrec = nullptr;     // the records of the chunks without F_LINKS, for the boundary tiles under fused()
+  uint32_t *rrnode = nullptr;
+  std::vector<uint32_t> rplane; // [nz + 1] first of them in each plane
   long long nb = 0, nl = 0, nfluid = 0;
   int has_uw = 0;
   int has_shell = 0;  // the static geometry has links across thin shells
@@ -90,22 +97,38 @@ struct lbm_sim {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // captured step loops, by starting buffer
   int2 *tiles = nullptr;      // step-kernel tile table (device)
   long long ntiles = 0;
-  int2 *btiles = nullptr;     // split step (variants 9, 10): the boundary entries (device)
+  int2 *btiles = nullptr;     // split(): the boundary entries (device)
   long long nbtiles = 0;
-  cudaStream_t aux = nullptr;                         // split step: the boundary kernel's stream
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;   // split step: orders aux around each step
+  cudaStream_t aux = nullptr;                         // split(): the boundary kernel's stream
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;   // split(): orders aux around each step
   int tiles_bx = 0, tiles_by = 0;  // launch shape the table was built for (0: stale)
   int tiles_per_block = 4;          // consecutive table entries per step-kernel block (1..4)
   int tiles_var = -1;               // register variant the launch data was prepared for
+  bool tiles_fused = false;         // fused() when the table was built
   int tma_blocks = 0, tma_smem = 0; // persistent grid and shared memory of the TMA-staged step
   int step_bx = 32, step_by = 8, variant = 0;
+  bool launch_set = false;  // by lbm_set_launch or lbm_autotune
   bool geom_ok = false, state_ok = false;
   int version = 0;  // bumped whenever the kernel view changes (options, geometry)
   MovingBody mb;
   std::string err;
 
   int npt() const { return variant >= 5 && variant <= 8 ? 2 : 1; }  // nodes per thread along x in lattice tiles
-  bool split() const { return variant == 9 || variant == 10; }      // lattice and boundary kernels apart
+  bool split() const { return variant == 9 || variant == 10 || fused(); }  // lattice and boundary kernels apart
+  // The bulk step: the one-node launches (variants 0..3, 11, 12, and the batched step's)
+  // where the rule is ELIBB-F or -FQ with the bounce-back wall estimate (bulk_row,
+  // warp_links). The other rules, thin shells and the other variants go through the
+  // tile table, as do lattices with more rows or planes than a grid has.
+  bool fused() const {
+    return !has_shell && wall_neq == LBM_NEQ_BOUNCE_BACK && (bc == LBM_BC_ELIBB_F || bc == LBM_BC_ELIBB_FQ) &&
+           (variant < 4 || variant == 11 || variant == 12) && ny <= 65535 && nz <= 65535;
+  }
+  // dynamic shared memory of a step kernel's block: the boundary tiles' staging (table
+  // or body entries present) and the warps' link staging
+  int step_smem(int threads, bool boundary_tiles, bool links) const {
+    const int a = boundary_tiles ? Q * threads : 0, b = links ? (Q + 5) * 32 * ((threads + 31) / 32) : 0;
+    return (a > b ? a : b) * (int)link_size();
+  }
   size_t elem_size() const;
   size_t link_size() const;
   void lattice_c(int i, int &x, int &y, int &z) const;
@@ -114,7 +137,8 @@ struct lbm_sim {
   lbm::Launch shape(int bx, int by) const;
   lbm::Launch step_shape() const;
   lbm::Launch aux_shape() const;
-  void tune_default();
+  void wide_shape();
+  void tune_default();  // the launch while !launch_set
   int ensure_scratch(long long doubles);
   void free_geometry();
   void drop_graphs();
@@ -126,6 +150,7 @@ struct lbm_sim {
   int capture(int parity);
   int upload(const lbm::HostGeometry &g);
   int download(lbm::HostGeometry &g);
+  int build_links();      // View::chunk and View::ldesc of the static geometry (geometry.cu)
   int finish_geometry();  // written-ahead masks and hash of the static geometry just set
   int ensure_stage_f();
 };

@@ -4,8 +4,9 @@
 // path, the TMA-staged kernel). They are compiled in three translation units per
 // (lattice, storage type), step_inst.cu built once for each part of each pair, so
 // that the build runs them in parallel: the one-node kernels (launch_one_ls), the
-// node pairs and the TMA-staged kernel (launch_wide_ls), the split step and the
-// batched step (launch_split_ls, launch_batch_ls). kernels.cu dispatches to them.
+// node pairs and the TMA-staged kernel (launch_wide_ls), and the bulk step with
+// the split and the batched step (launch_bulk_ls, launch_split_ls, launch_batch_ls). kernels.cu
+// dispatches to them.
 #pragma once
 
 #include "kernels.cuh"
@@ -22,32 +23,60 @@ cudaError_t step_variant(const View &v, const void *fin, void *fout, const Launc
   const S *a = static_cast<const S *>(fin);
   S *b = static_cast<S *>(fout);
   switch (phys_of(v)) {
-    case PH_FORCE: k_step<L, S, M, MINB, PH_FORCE, PAIR, MAXT><<<l.grid, l.block, 0, l.stream>>>(v, a, b); break;
-    case PH_TRT: k_step<L, S, M, MINB, PH_TRT, PAIR, MAXT><<<l.grid, l.block, 0, l.stream>>>(v, a, b); break;
+    case PH_FORCE: k_step<L, S, M, MINB, PH_FORCE, PAIR, MAXT><<<l.grid, l.block, l.smem, l.stream>>>(v, a, b); break;
+    case PH_TRT: k_step<L, S, M, MINB, PH_TRT, PAIR, MAXT><<<l.grid, l.block, l.smem, l.stream>>>(v, a, b); break;
     case PH_FORCE | PH_TRT:
-      k_step<L, S, M, MINB, PH_FORCE | PH_TRT, PAIR, MAXT><<<l.grid, l.block, 0, l.stream>>>(v, a, b);
+      k_step<L, S, M, MINB, PH_FORCE | PH_TRT, PAIR, MAXT><<<l.grid, l.block, l.smem, l.stream>>>(v, a, b);
       break;
-    default: k_step<L, S, M, MINB, 0, PAIR, MAXT><<<l.grid, l.block, 0, l.stream>>>(v, a, b); break;
+    default: k_step<L, S, M, MINB, 0, PAIR, MAXT><<<l.grid, l.block, l.smem, l.stream>>>(v, a, b); break;
   }
   return cudaGetLastError();
 }
 
-// The split step (variants 9, 10): the boundary kernel on lb.stream, then the
-// lattice kernel on l.stream. The caller orders the two streams around the pair.
+// The boundary kernel of the split and the bulk step, on lb->stream (where lb is given).
+// The caller orders the two streams around the pair of kernels.
+template <class L, typename S, typename M>
+cudaError_t boundary_launch(const View &v, const void *fin, void *fout, const Launch *lb) {
+  if (lb == nullptr || lb->grid.x == 0) return cudaSuccess;
+  k_boundary<L, S, M><<<lb->grid, lb->block, lb->smem, lb->stream>>>(v, static_cast<const S *>(fin),
+                                                                     static_cast<S *>(fout));
+  return cudaGetLastError();
+}
+
+// The split step (variants 9, 10): the boundary kernel, then the lattice kernel on l.stream.
 template <class L, typename S, typename M, int MINB>
 cudaError_t split_variant(const View &v, const void *fin, void *fout, const Launch &l, const Launch *lb) {
   const S *a = static_cast<const S *>(fin);
   S *b = static_cast<S *>(fout);
-  if (lb != nullptr && lb->grid.x > 0) {
-    k_boundary<L, S, M><<<lb->grid, lb->block, 0, lb->stream>>>(v, a, b);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e = boundary_launch<L, S, M>(v, fin, fout, lb);
+  if (e != cudaSuccess) return e;
   switch (phys_of(v)) {
     case PH_FORCE: k_lattice<L, S, M, MINB, PH_FORCE><<<l.grid, l.block, 0, l.stream>>>(v, a, b); break;
     case PH_TRT: k_lattice<L, S, M, MINB, PH_TRT><<<l.grid, l.block, 0, l.stream>>>(v, a, b); break;
     case PH_FORCE | PH_TRT: k_lattice<L, S, M, MINB, PH_FORCE | PH_TRT><<<l.grid, l.block, 0, l.stream>>>(v, a, b); break;
     default: k_lattice<L, S, M, MINB, 0><<<l.grid, l.block, 0, l.stream>>>(v, a, b); break;
+  }
+  return cudaGetLastError();
+}
+
+// The bulk step: the boundary kernel for what is left to it, then the bulk kernel, whose
+// grid is the lattice (l.grid: x tiles, groups of y tiles, planes).
+template <class L, typename S, typename M, int MINB>
+cudaError_t bulk_variant(const View &v, const void *fin, void *fout, const Launch &l, const Launch *lb) {
+  cudaError_t e = boundary_launch<L, S, M>(v, fin, fout, lb);
+  if (e != cudaSuccess) return e;
+  Planes p;
+  for (int i = 0; i < L::Q; ++i) {  // an integer sum: a shifted plane may begin before its buffer
+    p.src[i] = reinterpret_cast<const void *>(reinterpret_cast<uintptr_t>(fin) + (long long)v.loff[i] * (long long)sizeof(S));
+    p.dst[i] = static_cast<S *>(fout) + v.soff[i];
+  }
+  p.fin = fin;
+  p.fout = fout;
+  switch (phys_of(v)) {
+    case PH_FORCE: k_bulk<L, S, M, MINB, PH_FORCE><<<l.grid, l.block, l.smem, l.stream>>>(v, p); break;
+    case PH_TRT: k_bulk<L, S, M, MINB, PH_TRT><<<l.grid, l.block, l.smem, l.stream>>>(v, p); break;
+    case PH_FORCE | PH_TRT: k_bulk<L, S, M, MINB, PH_FORCE | PH_TRT><<<l.grid, l.block, l.smem, l.stream>>>(v, p); break;
+    default: k_bulk<L, S, M, MINB, 0><<<l.grid, l.block, l.smem, l.stream>>>(v, p); break;
   }
   return cudaGetLastError();
 }
@@ -130,6 +159,23 @@ cudaError_t launch_one_ls(int variant, const View &v, const void *fin, void *fou
   }
 }
 
+// The same variants as the bulk step (View::fused).
+template <class L, typename S>
+cudaError_t launch_bulk_ls(int variant, const View &v, const void *fin, void *fout, const Launch &l,
+                            const Launch *lb) {
+  using M = typename MathOf<S>::T;
+  if constexpr (sizeof(M) == 8) {
+    return bulk_variant<L, S, M, 1>(v, fin, fout, l, lb);
+  } else {
+    switch (variant) {
+      case 3: return bulk_variant<L, S, M, 4>(v, fin, fout, l, lb);
+      case 11: return bulk_variant<L, S, M, 5>(v, fin, fout, l, lb);
+      case 12: return bulk_variant<L, S, M, 6>(v, fin, fout, l, lb);
+      default: return bulk_variant<L, S, M, 3>(v, fin, fout, l, lb);
+    }
+  }
+}
+
 template <class L, typename S>
 cudaError_t launch_wide_ls(int variant, const View &v, const void *fin, void *fout, const Launch &l) {
   using M = typename MathOf<S>::T;
@@ -159,29 +205,60 @@ cudaError_t launch_split_ls(int variant, const View &v, const void *fin, void *f
   else return split_variant<L, S, M, 5>(v, fin, fout, l, lb);
 }
 
-// Batched step of the tiles of one physics class (l.grid.x blocks); variant 0..2: 80
-// registers, 3: 64.
-template <class L, typename S, typename M, int MINB>
-cudaError_t batch_variant(int phys, const BatchEntry *e, const int4 *tiles, int n, int T, int parity,
-                          const Launch &l) {
-  switch (phys) {
-    case PH_FORCE: k_step_batch<L, S, M, MINB, PH_FORCE><<<l.grid, l.block, 0, l.stream>>>(e, tiles, n, T, parity); break;
-    case PH_TRT: k_step_batch<L, S, M, MINB, PH_TRT><<<l.grid, l.block, 0, l.stream>>>(e, tiles, n, T, parity); break;
-    case PH_FORCE | PH_TRT:
-      k_step_batch<L, S, M, MINB, PH_FORCE | PH_TRT><<<l.grid, l.block, 0, l.stream>>>(e, tiles, n, T, parity);
-      break;
-    default: k_step_batch<L, S, M, MINB, 0><<<l.grid, l.block, 0, l.stream>>>(e, tiles, n, T, parity); break;
+// Kernels of the batched step for one physics class. FP64 on D3Q19 in blocks of 256
+// threads stages just 48 KB, which with a kernel's static copy of an entry passes the
+// default limit of 48 KB.
+template <class Kern>
+cudaError_t batch_kernel(Kern kern, const BatchEntry *e, const int4 *tiles, int n, int T, int parity,
+                         const Launch &l) {
+  if (l.smem + (int)(sizeof(BatchEntry) + sizeof(Planes)) > 48 * 1024) {
+    const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, l.smem);
+    if (r != cudaSuccess) return r;
   }
+  kern<<<l.grid, l.block, l.smem, l.stream>>>(e, tiles, n, T, parity);
   return cudaGetLastError();
 }
 
+template <class L, typename S, typename M, int MINB, bool BULK, int PHYS>
+cudaError_t batch_phys(const BatchEntry *e, const int4 *tiles, int n, int T, int parity, const Launch &l) {
+  if constexpr (BULK) return batch_kernel(k_bulk_batch<L, S, M, MINB, PHYS>, e, tiles, n, T, parity, l);
+  else return batch_kernel(k_step_batch<L, S, M, MINB, PHYS>, e, tiles, n, T, parity, l);
+}
+
+template <class L, typename S, typename M, int MINB, bool BULK>
+cudaError_t batch_variant(int phys, const BatchEntry *e, const int4 *tiles, int n, int T, int parity,
+                          const Launch &l) {
+  switch (phys) {
+    case PH_FORCE: return batch_phys<L, S, M, MINB, BULK, PH_FORCE>(e, tiles, n, T, parity, l);
+    case PH_TRT: return batch_phys<L, S, M, MINB, BULK, PH_TRT>(e, tiles, n, T, parity, l);
+    case PH_FORCE | PH_TRT: return batch_phys<L, S, M, MINB, BULK, PH_FORCE | PH_TRT>(e, tiles, n, T, parity, l);
+    default: return batch_phys<L, S, M, MINB, BULK, 0>(e, tiles, n, T, parity, l);
+  }
+}
+
+// kind: the tiles of the fused simulations (kBatchBulk), their boundary tiles
+// (kBatchBoundary, one per block), or the other simulations' tiles (kBatchStep).
+// Register budgets: bulk tiles 64, and 48 for variant 3; the other simulations' tiles
+// 80, and 64 for variant 3.
 template <class L, typename S>
-cudaError_t launch_batch_ls(int variant, int phys, const BatchEntry *e, const int4 *tiles, int n, int T,
+cudaError_t launch_batch_ls(int variant, int kind, int phys, const BatchEntry *e, const int4 *tiles, int n, int T,
                             int parity, const Launch &l) {
   using M = typename MathOf<S>::T;
-  if constexpr (sizeof(M) == 8) return batch_variant<L, S, M, 1>(phys, e, tiles, n, T, parity, l);
-  else if (variant == 3) return batch_variant<L, S, M, 4>(phys, e, tiles, n, T, parity, l);
-  else return batch_variant<L, S, M, 3>(phys, e, tiles, n, T, parity, l);
+  if (kind == kBatchBoundary) {
+    k_boundary_batch<L, S, M><<<l.grid, l.block, l.smem, l.stream>>>(e, tiles, parity);
+    return cudaGetLastError();
+  }
+  if constexpr (sizeof(M) == 8) {
+    if (kind == kBatchBulk) return batch_variant<L, S, M, 1, true>(phys, e, tiles, n, T, parity, l);
+    return batch_variant<L, S, M, 1, false>(phys, e, tiles, n, T, parity, l);
+  } else {
+    if (kind == kBatchBulk) {
+      if (variant == 3) return batch_variant<L, S, M, 5, true>(phys, e, tiles, n, T, parity, l);
+      return batch_variant<L, S, M, 4, true>(phys, e, tiles, n, T, parity, l);
+    }
+    if (variant == 3) return batch_variant<L, S, M, 4, false>(phys, e, tiles, n, T, parity, l);
+    return batch_variant<L, S, M, 3, false>(phys, e, tiles, n, T, parity, l);
+  }
 }
 
 template <class L, typename S>
@@ -210,9 +287,11 @@ cudaError_t prepare_step_tma_ls(int phys, int bx, int by, long long ntiles, int 
   X template cudaError_t launch_wide_ls<Lat, Sto>(int, const View &, const void *, void *, const Launch &); \
   X template cudaError_t prepare_step_tma_ls<Lat, Sto>(int, int, int, long long, int *, int *);
 #define LBM_STEP_PART2(X, Lat, Sto)                                                              \
+  X template cudaError_t launch_bulk_ls<Lat, Sto>(int, const View &, const void *, void *, const Launch &, \
+                                                   const Launch *);                              \
   X template cudaError_t launch_split_ls<Lat, Sto>(int, const View &, const void *, void *, const Launch &, \
                                                    const Launch *);                              \
-  X template cudaError_t launch_batch_ls<Lat, Sto>(int, int, const BatchEntry *, const int4 *, int, int, int, \
+  X template cudaError_t launch_batch_ls<Lat, Sto>(int, int, int, const BatchEntry *, const int4 *, int, int, int, \
                                                    const Launch &);
 #define LBM_STEP_DECLARE(Lat, Sto)      \
   LBM_STEP_PART0(extern, Lat, Sto)      \
