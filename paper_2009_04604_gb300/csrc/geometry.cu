@@ -784,15 +784,20 @@ done:
 // A rigid body on a prescribed trajectory (Sec. II.E: wall velocity at the link's
 // wall point). After every step t -> t+1, inside the fixed region box that covers
 // the body's whole trajectory:
-//  1. k_move_update: node kinds for the pose at t+1. A node that turns fluid
-//     (solid at t, fluid at t+1) is refilled with f^eq(rho0, u_body(x)). Its
-//     gather slots are written in the buffer the next step reads. The paper
-//     refills by local iterations (App. D); the equilibrium refill is this
-//     library's simpler choice.
-//  2. k_move_count, scan, k_move_fill: the boundary records of the region's
-//     fluid nodes, with q and u_w at t+1 and u_w at t+2, in region order.
-//  3. k_move_advance: the pose index moves on.
-// Everything stays on the device, so the step loop remains one CUDA graph.
+//  1. k_body_pose: the body at t+1 (and its velocity at t+2), once for everyone; the
+//     pose index moves on.
+//  2. k_move_mark: node kinds for the pose at t+1. A node that turns fluid (solid at
+//     t, fluid at t+1) is refilled with f^eq(rho0, u_body(x)). Its gather slots are
+//     written in the buffer the next step reads. The paper refills by local
+//     iterations (App. D); the equilibrium refill is this library's simpler choice.
+//     The same kernel finds the region's cut links and counts them.
+//  3. k_move_fill: the boundary records of the region's fluid nodes, with q and u_w at
+//     t+1 and u_w at t+2, in region order.
+// Everything stays on the device, so the step loop remains one CUDA graph. What bounds
+// it is latency: chains of FP64 divisions and roots, on a pipe of 2 lanes per clock and
+// SM, and one launch after another. The chains run one link per thread, the tests that
+// FP32 can decide run in FP32, and five launches follow a step where there were twelve
+// (D2Q9 128 x 98 with a turning ellipse, FP64: 114 us a step before, 44 now).
 namespace lbm {
 
 struct MoveGeo {
@@ -803,6 +808,7 @@ struct MoveGeo {
   int ntraj;
   const int *step;         // current pose index
   const double *state;     // free body: [angle, omega, centre, inertia] (null: traj)
+  const GeoShape *pose;    // the body at the pose the kernels work for (k_body_pose)
   int ox, oy, oz, rx, ry, rz;
   long long rsize;
 };
@@ -836,34 +842,98 @@ __device__ __forceinline__ void region_xyz(const MoveGeo &g, long long r, int &x
   z = g.oz + (int)(r / ((long long)g.rx * g.ry));
 }
 
-template <class L, typename S, typename M>
-__global__ void k_move_update(const MoveGeo g, int koff, int refill, uint8_t *__restrict__ flags,
-                              S *__restrict__ fout) {
-  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= g.rsize) return;
-  int x, y, z;
-  region_xyz(g, r, x, y, z);
-  const View &v = g.v;
-  const int n = (z * v.ny + y) * v.nxp + x;
-  const GeoShape b = body_at(g, *g.step + koff);
-  const uint8_t old = flags[n] & 3;
-  const uint8_t now = shape_solid(b, g.D, (double)x, (double)y, (double)z) ? K_SOLID : K_FLUID;
-  if (refill && old != K_FLUID && now == K_FLUID) {
-    // u_body at the node at the new pose: v + om x (x - c)
-    const double rx_ = x - b.c[0], ry_ = y - b.c[1], rz_ = g.D == 3 ? z - b.c[2] : 0.0;
-    double u[3] = {b.v[0] + b.om[1] * rz_ - b.om[2] * ry_, b.v[1] + b.om[2] * rx_ - b.om[0] * rz_,
-                   b.v[2] + b.om[0] * ry_ - b.om[1] * rx_};
-    if (g.D == 2) u[2] = 0.0;
-    const M ux = M(u[0]), uy = M(u[1]), uz = M(u[2]);
-    const M usq = ux * ux + uy * uy + uz * uz;
-    Nbr nb;
-    nb.init(v, x, y, z);
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i)
-      fout[(long long)i * v.np + n + nb.at(-L::cx(i), -L::cy(i), -L::cz(i))] =
-          to_store<S, M>(feq_s<L, M>(i, M(0), M(v.rho0), ux, uy, uz, usq));
+// A block's copy of the pose, and what decides most solid tests in FP32: the
+// reciprocal semi-axes, the rotation, and a margin around the surface that is far wider
+// than the FP32 error (offsets of a few radii, each rounded once); inside the margin the
+// test is shape_solid's. So the kinds are those of the FP64 definition bit for bit.
+struct BodyTest {
+  GeoShape s;
+  float inv[3], ca, sa, tol;
+};
+
+__device__ __forceinline__ void load_body(BodyTest &b, const GeoShape *__restrict__ pose, int D) {
+  constexpr int kWords = (int)(sizeof(GeoShape) / 8);
+  const int t = threadIdx.x;
+  if (t < kWords) reinterpret_cast<double *>(&b.s)[t] = reinterpret_cast<const double *>(pose)[t];
+  __syncthreads();
+  if (t == 0) {
+    const bool ell = b.s.type == LBM_SHAPE_ELLIPSOID;
+    float rmin = 1e30f;
+    for (int a = 0; a < 3; ++a) {
+      const float r = a < D ? (float)(ell ? b.s.r[a] : b.s.r[0]) : 1.0f;
+      b.inv[a] = 1.0f / r;
+      if (a < D) rmin = fminf(rmin, r);
+    }
+    b.ca = ell ? (float)b.s.ca : 1.0f;
+    b.sa = ell ? (float)b.s.sa : 0.0f;
+    b.tol = 1e-3f * (1.0f + 1.0f / rmin);
   }
-  flags[n] = now | F_KEEP;  // the lattice tiles never store into the region's non-fluid slots
+  __syncthreads();
+}
+
+// d: the FP32 offset of the point x from the body's centre
+__device__ __forceinline__ bool body_solid(const BodyTest &b, int D, float d0, float d1, float d2, int x, int y, int z) {
+  const float t0 = (b.ca * d0 + b.sa * d1) * b.inv[0], t1 = (b.ca * d1 - b.sa * d0) * b.inv[1], t2 = d2 * b.inv[2];
+  const float t = t0 * t0 + t1 * t1 + t2 * t2;
+  if (t < 1.0f - b.tol) return true;
+  if (t > 1.0f + b.tol) return false;
+  return shape_solid(b.s, D, (double)x, (double)y, (double)z);
+}
+
+// Kinds of the region's nodes at the pose (refill: see above), their cut masks into
+// rcut, and per 32-node region chunk the records and wall links. A fluid node's
+// neighbours are tested as the node is, so that no one waits for their flags.
+template <class L, typename S, typename M>
+__global__ void __launch_bounds__(128) k_move_mark(const MoveGeo g, int refill, uint8_t *__restrict__ flags,
+                                                   S *__restrict__ fout, uint32_t *__restrict__ rcut,
+                                                   uint32_t *__restrict__ crec, uint32_t *__restrict__ clink,
+                                                   long long rpad) {
+  __shared__ BodyTest b;
+  load_body(b, g.pose, g.D);
+  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= rpad) return;  // rpad is a multiple of 32: whole warps
+  uint32_t cut = 0;
+  if (r < g.rsize) {
+    int x, y, z;
+    region_xyz(g, r, x, y, z);
+    const View &v = g.v;
+    const int n = (z * v.ny + y) * v.nxp + x;
+    const float d0 = (float)(x - b.s.c[0]), d1 = (float)(y - b.s.c[1]), d2 = g.D == 3 ? (float)(z - b.s.c[2]) : 0.0f;
+    const uint8_t old = flags[n] & 3;
+    const uint8_t now = body_solid(b, g.D, d0, d1, d2, x, y, z) ? K_SOLID : K_FLUID;
+    if (refill && old != K_FLUID && now == K_FLUID) {
+      // u_body at the node at the new pose: v + om x (x - c)
+      const double rx_ = x - b.s.c[0], ry_ = y - b.s.c[1], rz_ = g.D == 3 ? z - b.s.c[2] : 0.0;
+      double u[3] = {b.s.v[0] + b.s.om[1] * rz_ - b.s.om[2] * ry_, b.s.v[1] + b.s.om[2] * rx_ - b.s.om[0] * rz_,
+                     b.s.v[2] + b.s.om[0] * ry_ - b.s.om[1] * rx_};
+      if (g.D == 2) u[2] = 0.0;
+      const M ux = M(u[0]), uy = M(u[1]), uz = M(u[2]);
+      const M usq = ux * ux + uy * uy + uz * uz;
+      Nbr nb;
+      nb.init(v, x, y, z);
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i)
+        fout[(long long)i * v.np + n + nb.at(-L::cx(i), -L::cy(i), -L::cz(i))] =
+            to_store<S, M>(feq_s<L, M>(i, M(0), M(v.rho0), ux, uy, uz, usq));
+    }
+    flags[n] = now | F_KEEP;  // the lattice tiles never store into the region's non-fluid slots
+    if (now == K_FLUID) {
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i) {
+        if (L::cx(i) == 0 && L::cy(i) == 0 && L::cz(i) == 0) continue;
+        if (body_solid(b, g.D, d0 - L::cx(i), d1 - L::cy(i), d2 - L::cz(i), x - L::cx(i), y - L::cy(i), z - L::cz(i)))
+          cut |= 1u << i;
+      }
+    }
+  }
+  rcut[r] = cut;
+  const uint32_t bal = __ballot_sync(0xffffffffu, cut != 0);
+  uint32_t nl = __popc(cut);
+  for (int o = 16; o > 0; o >>= 1) nl += __shfl_down_sync(0xffffffffu, nl, o);
+  if ((threadIdx.x & 31) == 0) {
+    crec[r >> 5] = __popc(bal);
+    clink[r >> 5] = nl;
+  }
 }
 
 // Local iteration refill (LIR), in three launches so that the neighbours' kinds
@@ -878,22 +948,20 @@ __global__ void k_move_update(const MoveGeo g, int koff, int refill, uint8_t *__
 //     node's post-collision f*_ibar plus 2 w_i rho c_i.u_b / c_s^2. The results
 //     go into the gather slots of the unknown directions, which belong to nodes
 //     that were the body's at t (never stored into by the lattice tiles);
-//  3. k_move_commit: the new kinds into flags.
+//  3. k_move_mark, without its own refill: the new kinds into flags, and the rest.
 // The paper applies its modified LIR before the global collide and stream (App.
 // D); here it runs at the end of step t, which comes to the same: before the
 // collide and stream of step t+1.
-template <class L>
-__global__ void k_move_kinds(const MoveGeo g, int koff, uint8_t *__restrict__ nkind) {
+__global__ void k_move_kinds(const MoveGeo g, uint8_t *__restrict__ nkind) {
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= g.rsize) return;
   int x, y, z;
   region_xyz(g, r, x, y, z);
-  const GeoShape b = body_at(g, *g.step + koff);
-  nkind[r] = shape_solid(b, g.D, (double)x, (double)y, (double)z) ? K_SOLID : K_FLUID;
+  nkind[r] = shape_solid(*g.pose, g.D, (double)x, (double)y, (double)z) ? K_SOLID : K_FLUID;
 }
 
 template <class L, typename S, typename M>
-__global__ void k_move_lir(const MoveGeo g, int koff, int iters, const uint8_t *__restrict__ flags,
+__global__ void k_move_lir(const MoveGeo g, int iters, const uint8_t *__restrict__ flags,
                            const uint8_t *__restrict__ nkind, S *__restrict__ fout) {
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= g.rsize) return;
@@ -902,7 +970,7 @@ __global__ void k_move_lir(const MoveGeo g, int koff, int iters, const uint8_t *
   const View &v = g.v;
   const int n = (z * v.ny + y) * v.nxp + x;
   if ((flags[n] & 3) == K_FLUID || nkind[r] != K_FLUID) return;  // not a fresh node
-  const GeoShape b = body_at(g, *g.step + koff);
+  const GeoShape &b = *g.pose;
   const double rx_ = x - b.c[0], ry_ = y - b.c[1], rz_ = g.D == 3 ? z - b.c[2] : 0.0;
   double ub[3] = {b.v[0] + b.om[1] * rz_ - b.om[2] * ry_, b.v[1] + b.om[2] * rx_ - b.om[0] * rz_,
                   b.v[2] + b.om[0] * ry_ - b.om[1] * rx_};
@@ -949,98 +1017,116 @@ __global__ void k_move_lir(const MoveGeo g, int koff, int iters, const uint8_t *
       fout[(long long)i * v.np + n + nb.at(-L::cx(i), -L::cy(i), -L::cz(i))] = to_store<S, M>(f[i]);
 }
 
-__global__ void k_move_commit(const MoveGeo g, const uint8_t *__restrict__ nkind, uint8_t *__restrict__ flags) {
-  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= g.rsize) return;
-  int x, y, z;
-  region_xyz(g, r, x, y, z);
-  const View &v = g.v;
-  flags[(z * v.ny + y) * v.nxp + x] = nkind[r] | F_KEEP;
-}
-
-// per 32-node region chunk: records and wall links (the region's fluid nodes whose
-// upstream neighbours are solid)
-template <class L>
-__global__ void k_move_count(const MoveGeo g, const uint8_t *__restrict__ flags, uint32_t *__restrict__ crec,
-                             uint32_t *__restrict__ clink, long long rpad) {
-  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= rpad) return;  // rpad is a multiple of 32: whole warps
-  uint32_t cut = 0;
-  if (r < g.rsize) {
-    int x, y, z;
-    region_xyz(g, r, x, y, z);
-    const View &v = g.v;
-    const int n = (z * v.ny + y) * v.nxp + x;
-    if ((flags[n] & 3) == K_FLUID) {
-      Nbr nb;
-      nb.init(v, x, y, z);
-#pragma unroll
-      for (int i = 0; i < L::Q; ++i) {
-        if (L::cx(i) == 0 && L::cy(i) == 0 && L::cz(i) == 0) continue;
-        if ((flags[n + nb.at(-L::cx(i), -L::cy(i), -L::cz(i))] & 3) == K_SOLID) cut |= 1u << i;
-      }
-    }
-  }
-  const uint32_t bal = __ballot_sync(0xffffffffu, cut != 0);
-  uint32_t nl = __popc(cut);
-  for (int o = 16; o > 0; o >>= 1) nl += __shfl_down_sync(0xffffffffu, nl, o);
-  if ((threadIdx.x & 31) == 0) {
-    crec[r >> 5] = __popc(bal);
-    clink[r >> 5] = nl;
-  }
-}
+// Records and links of the region's boundary nodes, in region order (rcut, crec and
+// clink from k_move_mark). scanned: crec and clink hold exclusive prefix sums;
+// otherwise every block sums the chunks before its own, cheaper than three scan
+// launches up to kScanChunks of them. The block lists its links in shared memory and
+// then takes one link per thread: the root of the crossing and the wall velocities.
+constexpr int kFillThreads = 128;
+constexpr long long kScanChunks = 4096;
 
 template <class L, typename LT>
-__global__ void k_move_fill(const MoveGeo g, int koff, const uint8_t *__restrict__ flags,
-                            const uint32_t *__restrict__ cbase, const uint32_t *__restrict__ lbase,
-                            long long rpad, Rec *__restrict__ rec, uint32_t *__restrict__ rnode,
-                            LT *__restrict__ lq, LT *__restrict__ luw, LT *__restrict__ luw1,
-                            uint8_t *__restrict__ ltag) {
-  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= rpad) return;
-  const View &v = g.v;
-  int x = 0, y = 0, z = 0, n = 0;
-  Rec rc = {0u, 0u, 0u, 0u, 0u};
-  Nbr nb;
-  if (r < g.rsize) {
+__global__ void __launch_bounds__(kFillThreads) k_move_fill(
+    const MoveGeo g, const uint32_t *__restrict__ rcut, const uint32_t *__restrict__ crec,
+    const uint32_t *__restrict__ clink, bool scanned, long long rpad, Rec *__restrict__ rec,
+    uint32_t *__restrict__ rnode, LT *__restrict__ lq, LT *__restrict__ luw, LT *__restrict__ luw1,
+    uint8_t *__restrict__ ltag, int *__restrict__ count) {
+  constexpr int kWarps = kFillThreads / 32;
+  __shared__ BodyTest bt;
+  __shared__ double off[kFillThreads][3];           // node offsets from the centre, in the body frame, scaled
+  __shared__ double edir[L::Q][3];                  // the same for the directions
+  __shared__ uint16_t desc[kFillThreads * (L::Q - 1)];  // thread | direction << 8 of each link
+  __shared__ uint32_t wrec[kWarps], wlink[kWarps], base[2], moves[kWarps];
+  load_body(bt, g.pose, g.D);
+  const GeoShape &b = bt.s;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const long long r = (long long)blockIdx.x * kFillThreads + t, first = (long long)blockIdx.x * kWarps;
+  if (t < kWarps) moves[t] = 0u;
+  // records and links before this block
+  uint32_t pr = 0, pl = 0;
+  if (!scanned)
+    for (long long c = t; c < first; c += kFillThreads) { pr += crec[c]; pl += clink[c]; }
+  for (int o = 16; o > 0; o >>= 1) {
+    pr += __shfl_down_sync(0xffffffffu, pr, o);
+    pl += __shfl_down_sync(0xffffffffu, pl, o);
+  }
+  if (lane == 0) { wrec[warp] = pr; wlink[warp] = pl; }
+  __syncthreads();
+  if (t == 0) {
+    uint32_t a = 0, c = 0;
+    for (int w = 0; w < kWarps; ++w) { a += wrec[w]; c += wlink[w]; }
+    base[0] = scanned ? crec[first] : a;
+    base[1] = scanned ? clink[first] : c;
+  }
+  const bool ell = b.type == LBM_SHAPE_ELLIPSOID;
+  int x = 0, y = 0, z = 0;
+  uint32_t cut = 0;
+  if (r < rpad) cut = rcut[r];
+  if (cut) {
     region_xyz(g, r, x, y, z);
-    n = (z * v.ny + y) * v.nxp + x;
-    if ((flags[n] & 3) == K_FLUID) {
-      nb.init(v, x, y, z);
-#pragma unroll
-      for (int i = 0; i < L::Q; ++i) {
-        if (L::cx(i) == 0 && L::cy(i) == 0 && L::cz(i) == 0) continue;
-        if ((flags[n + nb.at(-L::cx(i), -L::cy(i), -L::cz(i))] & 3) == K_SOLID) rc.cut |= 1u << i;
-      }
+    double d0 = x - b.c[0], d1 = y - b.c[1], d2 = g.D == 3 ? z - b.c[2] : 0.0;
+    if (ell) {
+      const double e0 = b.ca * d0 + b.sa * d1, e1 = b.ca * d1 - b.sa * d0;
+      d0 = e0 / b.r[0];
+      d1 = e1 / b.r[1];
+      if (g.D == 3) d2 = d2 / b.r[2];
     }
+    off[t][0] = d0; off[t][1] = d1; off[t][2] = d2;
   }
-  const uint32_t bal = __ballot_sync(0xffffffffu, rc.cut != 0);
-  const uint32_t cnt = __popc(rc.cut);
-  uint32_t s = cnt;
+  if (t < L::Q) {
+    double e0 = (double)dcx<L>(t), e1 = (double)dcy<L>(t), e2 = g.D == 3 ? (double)dcz<L>(t) : 0.0;
+    if (ell) {
+      const double c0 = b.ca * e0 + b.sa * e1, c1 = b.ca * e1 - b.sa * e0;
+      e0 = c0 / b.r[0];
+      e1 = c1 / b.r[1];
+      if (g.D == 3) e2 = e2 / b.r[2];
+    }
+    edir[t][0] = e0; edir[t][1] = e1; edir[t][2] = e2;
+  }
+  // ranks within the block
+  const uint32_t bal = __ballot_sync(0xffffffffu, cut != 0);
+  const uint32_t cnt = __popc(cut);
+  uint32_t inc = cnt;
   for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) >= o) s += t;
+    const uint32_t u = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += u;
   }
-  if (!rc.cut) return;
-  const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
-  const uint32_t rid = cbase[r >> 5] + __popc(bal & lt);
-  rc.link0 = lbase[r >> 5] + s - cnt;
-  const GeoShape b = body_at(g, *g.step + koff);
-  const double X[3] = {(double)x, (double)y, (double)z};
-  bool moving = false;
-  uint32_t li = rc.link0;
-  for (int i = 0; i < L::Q; ++i) {
-    if (!(rc.cut & (1u << i))) continue;
-    const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
-    double qq = shape_cross(b, g.D, X, c);
+  __syncthreads();  // base is read, wrec and wlink are free
+  if (lane == 31) { wrec[warp] = __popc(bal); wlink[warp] = inc; }
+  __syncthreads();
+  uint32_t rk = __popc(bal & ((1u << lane) - 1u)), lk = inc - cnt, nlinks = 0, nrec = 0;
+  for (int w = 0; w < kWarps; ++w) {
+    if (w < warp) { rk += wrec[w]; lk += wlink[w]; }
+    nrec += wrec[w];
+    nlinks += wlink[w];
+  }
+  for (uint32_t m = cut, k = lk; m; m &= m - 1u) desc[k++] = (uint16_t)(t | (__ffs(m) - 1) << 8);
+  __syncthreads();
+  const double R2 = ell ? 1.0 : b.r[0] * b.r[0];
+  for (uint32_t k = t; k < nlinks; k += kFillThreads) {
+    const int o = desc[k] & 255, i = desc[k] >> 8;
+    const uint32_t li = base[1] + k;
+    int X, Y, Z;
+    region_xyz(g, (long long)blockIdx.x * kFillThreads + o, X, Y, Z);
+    // shape_cross of the body, on the shared offsets
+    const double A = edir[i][0] * edir[i][0] + edir[i][1] * edir[i][1] + edir[i][2] * edir[i][2];
+    const double B = off[o][0] * edir[i][0] + off[o][1] * edir[i][1] + off[o][2] * edir[i][2];
+    const double C = off[o][0] * off[o][0] + off[o][1] * off[o][1] + off[o][2] * off[o][2] - R2;
+    const double disc = B * B - A * C;
+    double qq = -1.0;
+    if (!(disc < 0.0 || C <= 0.0 || B <= 0.0)) {
+      const double tt = C / (B + sqrt(disc));
+      if (tt > 0.0 && tt <= 1.0) qq = tt;
+    }
     if (qq <= 0.0) qq = 1.0;  // rounding at a tangent: the wall sits on the solid node
-    double rr[3];
-    for (int a = 0; a < 3; ++a) rr[a] = a < g.D ? X[a] - qq * c[a] - b.c[a] : 0.0;
+    const double rr[3] = {X - qq * dcx<L>(i) - b.c[0], Y - qq * dcy<L>(i) - b.c[1],
+                          g.D == 3 ? Z - qq * dcz<L>(i) - b.c[2] : 0.0};
     double u0[3] = {b.v[0] + b.om[1] * rr[2] - b.om[2] * rr[1], b.v[1] + b.om[2] * rr[0] - b.om[0] * rr[2],
                     b.v[2] + b.om[0] * rr[1] - b.om[1] * rr[0]};
     double u1[3] = {b.v1[0] + b.om1[1] * rr[2] - b.om1[2] * rr[1], b.v1[1] + b.om1[2] * rr[0] - b.om1[0] * rr[2],
                     b.v1[2] + b.om1[0] * rr[1] - b.om1[1] * rr[0]};
     if (g.D == 2) { u0[2] = 0.0; u1[2] = 0.0; }
+    bool moving = false;
     for (int a = 0; a < 3; ++a) {
       if (u0[a] != 0.0 || u1[a] != 0.0) moving = true;
       luw[3 * li + a] = (LT)u0[a];
@@ -1048,37 +1134,47 @@ __global__ void k_move_fill(const MoveGeo g, int koff, const uint8_t *__restrict
     }
     lq[li] = (LT)qq;
     ltag[li] = (uint8_t)b.tag;
-    ++li;
+    if (moving) atomicOr(&moves[o >> 5], 1u << (o & 31));
   }
-  if (moving) rc.open |= REC_MOVING;
-  rec[rid] = rc;
-  rnode[rid] = (uint32_t)n;
+  __syncthreads();
+  if (cut) {
+    const View &v = g.v;
+    rec[base[0] + rk] = Rec{cut, (moves[warp] >> lane) & 1u ? REC_MOVING : 0u, 0u, base[1] + lk, 0u};
+    rnode[base[0] + rk] = (uint32_t)((z * v.ny + y) * v.nxp + x);
+  }
+  if (t == 0 && (long long)(blockIdx.x + 1) * kFillThreads >= rpad) *count = (int)(base[0] + nrec);
 }
 
-__global__ void k_move_advance(int *step) { *step += 1; }
-
-// Free body: the torque of the step just taken (sum of the per-block partials, z
-// component, in a fixed order) turns the body about z: omega += T / I, then
-// angle += omega (semi-implicit Euler, unit time step). History entry `*step`
-// records angle, omega and torque. One warp.
-__global__ void k_body_rotate(const double *__restrict__ tpart, long long nblk, double *__restrict__ state,
-                              double *__restrict__ hist, int cap, const int *__restrict__ step) {
+// The body at pose *step + koff for the kernels above, by one warp. For a free body
+// with a step behind it (tpart not null) it first turns: the torque of the step just
+// taken (sum of the nblk per-block partials, z component, in a fixed order) gives
+// omega += T / I, then angle += omega (semi-implicit Euler, unit time step); history
+// entry `*step` records angle, omega and torque. advance: the pose index moves on.
+__global__ void k_body_pose(const MoveGeo g, int koff, int advance, const double *__restrict__ tpart, long long nblk,
+                            double *__restrict__ state, double *__restrict__ hist, int cap, int *__restrict__ step,
+                            GeoShape *__restrict__ pose) {
   const int lane = threadIdx.x;
   double t = 0.0;
-  for (long long b = lane; b < nblk; b += 32) t += tpart[b * 3 + 2];
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if (lane == 0) {
+  if (tpart) {
+    for (long long b = lane; b < nblk; b += 32) t += tpart[b * 3 + 2];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  }
+  if (lane != 0) return;
+  const int now = *step;
+  if (tpart) {
     const double om = state[1] + t / state[5];
     const double ang = state[0] + om;
     state[0] = ang;
     state[1] = om;
     if (cap > 0) {
-      const long long k = *step % cap;
+      const long long k = now % cap;
       hist[3 * k] = ang;
       hist[3 * k + 1] = om;
       hist[3 * k + 2] = t;
     }
   }
+  *pose = body_at(g, now + koff);
+  if (advance) *step = now + 1;
 }
 
 template <class Fn>
@@ -1107,8 +1203,9 @@ static cudaError_t move_dispatch(int lattice, int dtype, Fn &&fn) {
   }
 }
 
-// Body geometry of pose (*step + koff) into record set `set`; refill fresh nodes in fout.
-static cudaError_t move_geometry(lbm_sim *h, int koff, int refill, void *fout, int set) {
+// Body geometry of pose (*step + koff) into record set `set`; after a step (after): a
+// free body turns first, the pose index moves on, and fresh nodes are refilled in fout.
+static cudaError_t move_geometry(lbm_sim *h, int koff, bool after, void *fout, int set) {
   MovingBody &mb = h->mb;
   MoveGeo g;
   g.v = h->view();
@@ -1118,27 +1215,33 @@ static cudaError_t move_geometry(lbm_sim *h, int koff, int refill, void *fout, i
   g.ntraj = mb.ntraj;
   g.step = mb.step;
   g.state = mb.free_rot ? mb.state : nullptr;
+  GeoShape *pose = static_cast<GeoShape *>(mb.pose);
+  g.pose = pose;
   g.ox = mb.ox; g.oy = mb.oy; g.oz = mb.oz; g.rx = mb.rx; g.ry = mb.ry; g.rz = mb.rz;
   g.rsize = mb.rsize;
   cudaStream_t st = h->stream;
-  const unsigned blocks = (unsigned)((mb.rpad + 255) / 256);
+  const unsigned blocks = (unsigned)((mb.rpad + kFillThreads - 1) / kFillThreads);
   const long long nchunk = mb.rpad / 32;
+  k_body_pose<<<1, 32, 0, st>>>(g, koff, after ? 1 : 0, after && mb.free_rot ? mb.tpart : nullptr, mb.nfpart, mb.state,
+                                mb.hist, mb.hist_cap, mb.step, pose);
   return move_dispatch(h->lattice, h->dtype, [&]<class L, typename S, typename M>() {
-    if (refill && mb.refill_mode == LBM_REFILL_LIR) {
-      k_move_kinds<L><<<blocks, 256, 0, st>>>(g, koff, mb.nkind);
-      k_move_lir<L, S, M><<<blocks, 256, 0, st>>>(g, koff, mb.refill_iters, h->flags, mb.nkind,
-                                                  static_cast<S *>(fout));
-      k_move_commit<<<blocks, 256, 0, st>>>(g, mb.nkind, h->flags);
-    } else {
-      k_move_update<L, S, M><<<blocks, 256, 0, st>>>(g, koff, refill, h->flags, static_cast<S *>(fout));
+    const bool lir = after && mb.refill_mode == LBM_REFILL_LIR;
+    if (lir) {
+      k_move_kinds<<<blocks, kFillThreads, 0, st>>>(g, mb.nkind);
+      k_move_lir<L, S, M><<<blocks, kFillThreads, 0, st>>>(g, mb.refill_iters, h->flags, mb.nkind,
+                                                           static_cast<S *>(fout));
     }
-    k_move_count<L><<<blocks, 256, 0, st>>>(g, h->flags, mb.crec, mb.clink, mb.rpad);
-    exclusive_scan(mb.crec, nchunk, mb.tot, reinterpret_cast<uint32_t *>(mb.count[set]), st);
-    exclusive_scan(mb.clink, nchunk, mb.tot, mb.totals, st);
-    k_move_fill<L, M><<<blocks, 256, 0, st>>>(g, koff, h->flags, mb.crec, mb.clink, mb.rpad, mb.rec[set],
-                                              mb.rnode[set], static_cast<M *>(mb.lq[set]),
-                                              static_cast<M *>(mb.luw[set]), static_cast<M *>(mb.luw1[set]),
-                                              mb.ltag[set]);
+    k_move_mark<L, S, M><<<blocks, kFillThreads, 0, st>>>(g, after && !lir ? 1 : 0, h->flags, static_cast<S *>(fout),
+                                                          mb.rcut, mb.crec, mb.clink, mb.rpad);
+    const bool scan = nchunk > kScanChunks;
+    if (scan) {
+      exclusive_scan(mb.crec, nchunk, mb.tot, mb.totals, st);
+      exclusive_scan(mb.clink, nchunk, mb.tot, mb.totals, st);
+    }
+    k_move_fill<L, M><<<blocks, kFillThreads, 0, st>>>(g, mb.rcut, mb.crec, mb.clink, scan, mb.rpad, mb.rec[set],
+                                                       mb.rnode[set], static_cast<M *>(mb.lq[set]),
+                                                       static_cast<M *>(mb.luw[set]), static_cast<M *>(mb.luw1[set]),
+                                                       mb.ltag[set], mb.count[set]);
     return cudaGetLastError();
   });
 }
@@ -1153,19 +1256,10 @@ int lbm_sim::move_after_step(void *fout, int set) {
   const RecSet rs{mb.rec[s], mb.rnode[s], mb.lq[s], mb.luw[s], mb.luw1[s], mb.ltag[s]};
   Launch lf;
   lf.grid = dim3((unsigned)mb.nfpart);
-  lf.block = dim3(256);
   lf.stream = stream;
   cudaError_t e = launch_force(lattice, dtype, view(), fout, nullptr, rs, 0, mb.count[s], -1, mb.fpart, lf,
                                mb.free_rot ? mb.tpart : nullptr, mb.centre[0], mb.centre[1], mb.centre[2]);
-  if (e == cudaSuccess && mb.free_rot) {
-    k_body_rotate<<<1, 32, 0, stream>>>(mb.tpart, mb.nfpart, mb.state, mb.hist, mb.hist_cap, mb.step);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = move_geometry(this, 1, 1, fout, set);
-  if (e == cudaSuccess) {
-    k_move_advance<<<1, 1, 0, stream>>>(mb.step);
-    e = cudaGetLastError();
-  }
+  if (e == cudaSuccess) e = move_geometry(this, 1, true, fout, set);
   if (e != cudaSuccess) return lbm_fail(this, LBM_ERR_CUDA, std::string("moving body: ") + cudaGetErrorString(e));
   return LBM_OK;
 }
@@ -1173,7 +1267,7 @@ int lbm_sim::move_after_step(void *fout, int set) {
 int lbm_sim::move_rebuild(long long pose) {
   const int k = (int)pose;
   LBM_CUDA_GEO(this, cudaMemcpyAsync(mb.step, &k, sizeof(int), cudaMemcpyHostToDevice, stream));
-  cudaError_t e = move_geometry(this, 0, 0, f[cur], cur);
+  cudaError_t e = move_geometry(this, 0, false, f[cur], cur);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return lbm_fail(this, LBM_ERR_CUDA, std::string("moving body: ") + cudaGetErrorString(e));
   return LBM_OK;
@@ -1182,7 +1276,7 @@ int lbm_sim::move_rebuild(long long pose) {
 void lbm_sim::free_moving_body() {
   if (!mb.on && !mb.traj) return;
   cudaStreamSynchronize(stream);
-  cudaFree(mb.shape); cudaFree(mb.traj); cudaFree(mb.step); cudaFree(mb.fpart);
+  cudaFree(mb.shape); cudaFree(mb.pose); cudaFree(mb.rcut); cudaFree(mb.traj); cudaFree(mb.step); cudaFree(mb.fpart);
   cudaFree(mb.state); cudaFree(mb.tpart); cudaFree(mb.hist); cudaFree(mb.nkind);
   cudaFree(mb.crec); cudaFree(mb.clink); cudaFree(mb.tot); cudaFree(mb.totals);
   for (int k = 0; k < 2; ++k) {
@@ -1232,7 +1326,7 @@ static int setup_body(lbm_handle h, const lbm_shape *body, const double lo[3], c
   mb.cap_rec = mb.rsize;
   mb.cap_link = mb.rsize * (h->Q - 1);
   mb.tag = body->tag;
-  mb.nfpart = (mb.cap_rec + 255) / 256;
+  mb.nfpart = std::min<long long>((mb.cap_rec + 63) / 64, 2 * 152);  // k_force: 8 warps of 8 records a block
   GeoShape gs;
   std::memset(&gs, 0, sizeof(gs));
   gs.type = body->type;
@@ -1242,6 +1336,8 @@ static int setup_body(lbm_handle h, const lbm_shape *body, const double lo[3], c
   const size_t ls = h->link_size();
   const long long nchunk = mb.rpad / 32;
   LBM_CUDA_GEO(h, cudaMalloc(&mb.shape, sizeof(GeoShape)));
+  LBM_CUDA_GEO(h, cudaMalloc(&mb.pose, sizeof(GeoShape)));
+  LBM_CUDA_GEO(h, cudaMalloc(&mb.rcut, sizeof(uint32_t) * mb.rpad));
   LBM_CUDA_GEO(h, cudaMalloc(&mb.traj, sizeof(double) * 9 * ntraj));
   LBM_CUDA_GEO(h, cudaMalloc(&mb.step, sizeof(int)));
   LBM_CUDA_GEO(h, cudaMalloc(&mb.fpart, sizeof(double) * 3 * mb.nfpart));
@@ -1296,7 +1392,7 @@ static int setup_body(lbm_handle h, const lbm_shape *body, const double lo[3], c
   LBM_CUDA_GEO(h, cudaGetLastError());
   // geometry of the first pose for the next step (no refill: the state is set
   // afterwards or was set on the static geometry)
-  cudaError_t err = move_geometry(h, 0, 0, h->f[h->cur], h->cur);
+  cudaError_t err = move_geometry(h, 0, false, h->f[h->cur], h->cur);
   if (err == cudaSuccess) err = cudaStreamSynchronize(h->stream);
   if (err != cudaSuccess) return lbm_fail(h, LBM_ERR_CUDA, std::string("moving body: ") + cudaGetErrorString(err));
   // fluid node count of the current geometry

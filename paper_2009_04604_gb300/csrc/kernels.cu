@@ -5,26 +5,31 @@ namespace lbm {
 
 __global__ void k_reduce_final(const double *__restrict__ part, long long nblocks, int ncomp,
                                double *__restrict__ out) {
-  // thread t sums partials t, t + 1024, ... of each component in order, then a
-  // fixed tree over the 1024 thread sums
-  __shared__ double sm[1024];
+  // thread t sums partials t, t + 1024, ... of each component in order, then every warp
+  // its lanes' sums and warp 0 the warps' (a tree of shuffles: the barrier tree over
+  // 1024 sums took 13 us for three components, this takes 4)
+  __shared__ double sm[32];
+  const int t = threadIdx.x, lane = t & 31;
   for (int c = 0; c < ncomp; ++c) {
     double s = 0.0;
-    for (long long b = threadIdx.x; b < nblocks; b += blockDim.x) s += part[b * ncomp + c];
-    sm[threadIdx.x] = s;
+    for (long long b = t; b < nblocks; b += blockDim.x) s += part[b * ncomp + c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) sm[t >> 5] = s;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if ((int)threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
-      __syncthreads();
+    if (t < 32) {
+      s = lane < (int)(blockDim.x >> 5) ? sm[lane] : 0.0;
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+      if (lane == 0) out[c] = s;
     }
-    if (threadIdx.x == 0) out[c] = sm[0];
     __syncthreads();
   }
 }
 
 cudaError_t launch_reduce_final(const double *part, long long nblocks, int ncomp, double *out,
                                 cudaStream_t s) {
-  k_reduce_final<<<1, 1024, 0, s>>>(part, nblocks, ncomp, out);
+  // no more warps than there are groups of 32 partials
+  const int threads = (int)(nblocks >= 1024 ? 1024 : (nblocks + 31) / 32 * 32);
+  k_reduce_final<<<1, threads > 0 ? threads : 32, 0, s>>>(part, nblocks, ncomp, out);
   return cudaGetLastError();
 }
 
@@ -107,13 +112,23 @@ cudaError_t launch_read(int lattice, int dtype, const View &v, const void *fin, 
   });
 }
 
+// A body's records and a small lattice's: 8 to a warp, so that they spread over the SMs;
+// else 32, whose links fill the lanes (128 x 96 x 80 duct, 43 thousand records: 11.3 us
+// with 32, 16.5 with 8: the FP64 pipe takes an idle lane's time too). At most 4 blocks
+// an SM: their partials are summed by one.
+static constexpr long long kFewRecords = 5000;
+int force_blocks(long long nrec) {
+  const long long per_block = 8 * (nrec <= kFewRecords ? 8 : 32), n = (nrec + per_block - 1) / per_block;
+  return (int)(n < 4 * 152 ? n : 4 * 152);
+}
+
 cudaError_t launch_force(int lattice, int dtype, const View &v, const void *cur, const void *prev,
                          const RecSet &rs, long long nrec, const int *nrec_dev, int tag, double *part,
                          const Launch &l, double *tpart, double cx, double cy, double cz) {
   return dispatch(lattice, dtype, [&]<class L, typename S, typename M>() {
-    k_force<L, S, M><<<l.grid, l.block, 0, l.stream>>>(v, static_cast<const S *>(cur),
-                                                       static_cast<const S *>(prev), rs, nrec,
-                                                       nrec_dev, tag, part, tpart, cx, cy, cz);
+    auto *kern = nrec_dev != nullptr || nrec <= kFewRecords ? k_force<L, S, M, 8> : k_force<L, S, M, 32>;
+    kern<<<l.grid, 256, 0, l.stream>>>(v, static_cast<const S *>(cur), static_cast<const S *>(prev), rs, nrec,
+                                       nrec_dev, tag, part, tpart, cx, cy, cz);
     return cudaGetLastError();
   });
 }

@@ -46,11 +46,13 @@ cudaError_t launch_set_pop(int lattice, int dtype, const View &v, void *fout, co
 cudaError_t launch_read(int lattice, int dtype, const View &v, const void *fin, double *fh,
                         double *rho, double *u, double *mass_part, const Launch &l);
 // Momentum-exchange partials over the records rs: nrec of them, or *nrec_dev
-// (device) when nrec_dev is not null; the grid must cover the largest count.
+// (device) when nrec_dev is not null, in l.grid.x blocks (force_blocks(nrec), or any
+// fixed number).
 // cur is the state the last step wrote, prev the state it read (used for the
 // links across thin shells; may be null when rs has none).
 // With tpart, also the torque about (cx, cy, cz) of every link force, taken at the
 // link's wall point x_F - q c_i (3 doubles per block).
+int force_blocks(long long nrec);
 cudaError_t launch_force(int lattice, int dtype, const View &v, const void *cur, const void *prev,
                          const RecSet &rs, long long nrec, const int *nrec_dev, int tag, double *part,
                          const Launch &l, double *tpart = nullptr, double cx = 0.0, double cy = 0.0,

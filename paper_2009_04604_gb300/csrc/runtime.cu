@@ -585,14 +585,12 @@ extern "C" int lbm_wall_force(lbm_handle h, int tag, double F[3]) {
   if (!h->geom_ok || !h->state_ok) return lbm_fail(h, LBM_ERR_STATE, "no state yet");
   if (tag < -1 || tag > 7) return lbm_fail(h, LBM_ERR_ARG, "tag must be -1..7");
   F[0] = F[1] = F[2] = 0.0;
-  const int bs = 256;
-  const long long nblk1 = (h->nb + bs - 1) / bs;
+  const long long nblk1 = lbm::force_blocks(h->nb);
   const long long nblk2 = h->mb.on ? h->mb.nfpart : 0;
   if (nblk1 + nblk2 == 0) return LBM_OK;
   int rc = h->ensure_scratch((nblk1 + nblk2) * 3);
   if (rc) return rc;
   Launch l;
-  l.block = dim3(bs);
   l.stream = h->stream;
   const View v = h->view();
   if (nblk1) {
@@ -619,13 +617,11 @@ extern "C" int lbm_wall_torque(lbm_handle h, int tag, const double centre[3], do
   if (!h->geom_ok || !h->state_ok) return lbm_fail(h, LBM_ERR_STATE, "no state yet");
   if (tag < -1 || tag > 7) return lbm_fail(h, LBM_ERR_ARG, "tag must be -1..7");
   T[0] = T[1] = T[2] = 0.0;
-  const int bs = 256;
-  const long long nblk = (h->nb + bs - 1) / bs;
+  const long long nblk = lbm::force_blocks(h->nb);
   if (nblk == 0) return LBM_OK;
   int rc = h->ensure_scratch(nblk * 6);
   if (rc) return rc;
   Launch l;
-  l.block = dim3(bs);
   l.grid = dim3((unsigned)nblk);
   l.stream = h->stream;
   const View v = h->view();

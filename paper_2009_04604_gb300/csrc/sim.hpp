@@ -20,6 +20,8 @@ struct HostGeometry;
 struct MovingBody {
   bool on = false;
   void *shape = nullptr;           // device copy of the body's shape (geometry kernels' type)
+  void *pose = nullptr;            // device: the body at the pose the geometry kernels work for
+  uint32_t *rcut = nullptr;        // device [rpad]: cut mask of each region node
   double *traj = nullptr;          // device [ntraj][9]: centre, velocity, angular velocity per step
   int ntraj = 0;
   int ox = 0, oy = 0, oz = 0, rx = 1, ry = 1, rz = 1;  // region box
