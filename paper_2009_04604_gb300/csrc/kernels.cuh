@@ -879,6 +879,40 @@ __device__ __forceinline__ void warp_links(const View &v, const uint4 ck, const 
 }
 
 // ---------------------------------------------------------------- bulk tiles
+// Element step from the source of population i to that of population i + 1: a plane
+// further, at the next velocity. D3Q19 has four different steps, D3Q27 three, D2Q9 two.
+template <class L>
+__device__ __forceinline__ int source_step(int i, int np, int nxp, int plane) {
+  return np - (L::cx(i + 1) - L::cx(i)) - (L::cy(i + 1) - L::cy(i)) * nxp - (L::cz(i + 1) - L::cz(i)) * plane;
+}
+
+// The batched kernel's addresses. Its view lies in shared memory, where a pointer per
+// plane costs as many loads again as the populations do (k_bulk_batch at 70 % of the L1
+// throughput), so it walks the planes: sources 0 .. Q-1 in order, then the stores in
+// relax's order (the rest population, then the pairs i, Q-1-i). 16 FP16 ducts: 449 us a
+// step with the table, 441 walking; 96 small FP32 ducts 164 and 158.
+template <class L, typename S>
+struct WalkPlanes {
+  const S *fin;
+  S *fout;
+  int n, np, nxp, plane, at, up, down;
+  __device__ __forceinline__ WalkPlanes(const View &v, const Planes &pl, int node)
+      : fin(static_cast<const S *>(pl.fin)), fout(static_cast<S *>(pl.fout)), n(node), np((int)v.np), nxp(v.nxp),
+        plane(v.nxp * v.ny), at(node - (L::cx(0) + L::cy(0) * v.nxp + L::cz(0) * v.nxp * v.ny)), up(node),
+        down(node + (L::Q - 1) * (int)v.np) {}
+  __device__ __forceinline__ const S *src(int i, int wrap) {
+    const S *r = fin + (unsigned)(at + wrap);
+    if (i < L::Q - 1) at += source_step<L>(i, np, nxp, plane);
+    return r;
+  }
+  __device__ __forceinline__ S *dst(int i) {
+    if (i == L::Q / 2) return fout + (unsigned)(n + i * np);
+    S *r = fout + (unsigned)(i < L::Q / 2 ? up : down);
+    if (i < L::Q / 2) up += np; else down -= np;
+    return r;
+  }
+};
+
 // One row of a bulk tile: this warp's chunk of row (y, z). The step's instruction
 // count, not memory, bounds FP16 storage and the porous medium (74-77 % of the issue
 // slots taken; 565 and 960 instructions a warp through the tile table and the flags,
@@ -890,13 +924,14 @@ __device__ __forceinline__ void warp_links(const View &v, const uint4 ck, const 
 //    sources of c_x = +1 and -1 are addressed through an index of their own that
 //    carries the wrap of the lane at the row's end. Only rows at the y and z edges,
 //    and sheared row ends, gather through the wrap table.
-// Every plane has its own pointer (Planes), a constant operand, so that an address is
-// one multiply-add. Walking the planes instead, by 64-bit or by 32-bit steps, takes 10 %
-// more instructions and was slower (porous FP16, 192^3: 206 and 204 against 187 us).
+// In the single simulation's kernel every plane has its own pointer (Planes), a constant
+// operand, so that an address is one multiply-add. Walking the planes instead (WALK, the
+// batched kernel) takes 10 % more instructions there and was slower (porous FP16,
+// 192^3: 204 against 187 us).
 // A non-fluid node whose 32-byte sector holds a fluid node stores the relaxation of
 // zeros into the planes that take no written-ahead value, as in lattice_tile. The
 // nodes' arithmetic is lattice_tile's, operation for operation.
-template <class L, typename S, typename M, int PHYS, bool LINKS>
+template <class L, typename S, typename M, int PHYS, bool WALK>
 __device__ __forceinline__ void bulk_row(const View &v, const Planes &p, M *st, int x, int y, int z) {
   using U = Units<S>;
   const int n = (z * v.ny + y) * v.nxp + x;
@@ -904,15 +939,23 @@ __device__ __forceinline__ void bulk_row(const View &v, const Planes &p, M *st, 
   if (ck.w & CK_IDLE) return;
   const S *fin = static_cast<const S *>(p.fin);
   S *fout = static_cast<S *>(p.fout);
+  const bool links = (ck.w & CK_LINKS) != 0;
   const unsigned un = (unsigned)n;
-  const bool links = LINKS && (ck.w & CK_LINKS);
+  WalkPlanes<L, S> walk(v, p, n);
+  const auto dst = [&](int i) {
+    if constexpr (WALK) return walk.dst(i);
+    else return static_cast<S *>(p.dst[i]) + un;
+  };
   M f[L::Q];
   if ((ck.w & CK_PLAIN) && !links) {
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) f[i] = U::template load<M>(LD_POP(v, fin, static_cast<const S *>(p.src[i]) + un));
+    for (int i = 0; i < L::Q; ++i) {
+      if constexpr (WALK) f[i] = U::template load<M>(LD_POP(v, fin, walk.src(i, 0)));
+      else f[i] = U::template load<M>(LD_POP(v, fin, static_cast<const S *>(p.src[i]) + un));
+    }
     const Macro<L, M> m = moments<L, M, U::kStored>(v, f);
     relax<L, M, PHYS, U::kStored>(v, f, m, [&](int i, M val) {
-      ST_POP(v, fout, static_cast<S *>(p.dst[i]) + un, U::template store<M>(val));
+      ST_POP(v, fout, dst(i), U::template store<M>(val));
     });
     return;
   }
@@ -925,11 +968,16 @@ __device__ __forceinline__ void bulk_row(const View &v, const Planes &p, M *st, 
   uint32_t skip = 0;
   if (here) {
     if (rows_inside && (v.xshift == 0 || (x > 0 && x < v.nx - 1))) {
-      const unsigned up = un + (x == 0 ? v.nx : 0), dn = un - (x == v.nx - 1 ? v.nx : 0);
+      const int wu = x == 0 ? v.nx : 0, wd = x == v.nx - 1 ? -v.nx : 0;
+      const unsigned up = un + wu, dn = un + wd;
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i)
-        f[i] = U::template load<M>(
-            LD_POP(v, fin, static_cast<const S *>(p.src[i]) + (L::cx(i) > 0 ? up : (L::cx(i) < 0 ? dn : un))));
+      for (int i = 0; i < L::Q; ++i) {
+        if constexpr (WALK)
+          f[i] = U::template load<M>(LD_POP(v, fin, walk.src(i, L::cx(i) > 0 ? wu : (L::cx(i) < 0 ? wd : 0))));
+        else
+          f[i] = U::template load<M>(
+              LD_POP(v, fin, static_cast<const S *>(p.src[i]) + (L::cx(i) > 0 ? up : (L::cx(i) < 0 ? dn : un))));
+      }
     } else {
       Nbr nb;
       nb.init(v, x, y, z);
@@ -952,7 +1000,7 @@ __device__ __forceinline__ void bulk_row(const View &v, const Planes &p, M *st, 
   }
   if (here || fill) {
     const Macro<L, M> m = moments<L, M, U::kStored>(v, f);
-    if (LINKS && (fl & F_LINKS)) {
+    if (fl & F_LINKS) {
       M *col = st + (threadIdx.x & 31);
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) col[i * 32] = f[i];
@@ -964,11 +1012,16 @@ __device__ __forceinline__ void bulk_row(const View &v, const Planes &p, M *st, 
     }
     if (masked)
       relax<L, M, PHYS, U::kStored>(v, f, m, [&](int i, M val) {
-        if (!((skip >> i) & 1u)) ST_POP(v, fout, static_cast<S *>(p.dst[i]) + un, U::template store<M>(val));
+        if constexpr (WALK) {
+          S *to = dst(i);  // a walking address moves on in any case
+          if (!((skip >> i) & 1u)) ST_POP(v, fout, to, U::template store<M>(val));
+        } else {
+          if (!((skip >> i) & 1u)) ST_POP(v, fout, dst(i), U::template store<M>(val));
+        }
       });
     else
       relax<L, M, PHYS, U::kStored>(v, f, m, [&](int i, M val) {
-        ST_POP(v, fout, static_cast<S *>(p.dst[i]) + un, U::template store<M>(val));
+        ST_POP(v, fout, dst(i), U::template store<M>(val));
       });
   }
   if (links) {
@@ -1226,7 +1279,7 @@ __global__ void __launch_bounds__(256, MINB) k_bulk(const __grid_constant__ View
   int y = blockIdx.y * T * blockDim.y + threadIdx.y;
 #pragma unroll 1
   for (int k = 0; k < T; ++k, y += blockDim.y)
-    if (y < v.ny) bulk_row<L, S, M, PHYS, true>(v, p, st, x, y, blockIdx.z);
+    if (y < v.ny) bulk_row<L, S, M, PHYS, false>(v, p, st, x, y, blockIdx.z);
 }
 
 // ---------------------------------------------------------------- TMA-staged step
@@ -1511,27 +1564,32 @@ __global__ void __launch_bounds__(256, MINB) k_bulk_batch(const BatchEntry *__re
                                                           const int4 *__restrict__ tiles, int ntiles,
                                                           int T, int parity) {
   __shared__ BatchEntry se;
-  __shared__ Planes pl;
   const int t = threadIdx.y * blockDim.x + threadIdx.x;
   M *st = step_stage<M>() + (t >> 5) * (kStageRows<L> * 32);
   int held = -1;
+  Planes pl;  // the two buffers
   for (int k = 0; k < T; ++k) {
     const int idx = blockIdx.x * T + k;
     if (idx >= ntiles) break;  // uniform across the block
     const int4 tile = tiles[idx];
     if (hold_entry(se, entries, tile.x, held)) {
-      if (t < L::Q) {
-        pl.src[t] = static_cast<const S *>(parity ? se.f1 : se.f0) + se.v.loff[t];
-        pl.dst[t] = static_cast<S *>(parity ? const_cast<void *>(se.f0) : se.f1) + se.v.soff[t];
-      }
-      if (t == 0) {
-        pl.fin = parity ? se.f1 : se.f0;
-        pl.fout = parity ? const_cast<void *>(se.f0) : se.f1;
-      }
-      __syncthreads();
+      pl.fin = parity ? se.f1 : se.f0;
+      pl.fout = parity ? const_cast<void *>(se.f0) : se.f1;
     }
-    const int y = tile.w * blockDim.y + threadIdx.y;
-    if (y < se.v.ny) bulk_row<L, S, M, PHYS, true>(se.v, pl, st, tile.z * blockDim.x + threadIdx.x, y, tile.y);
+    const int x = tile.z * blockDim.x + threadIdx.x, y = tile.w * blockDim.y + threadIdx.y;
+    // what the next tile asks for first, its chunk and flags, meanwhile: tiles follow one
+    // another along x, then y, then z, and the loads of one depend on each other
+    if (k + 1 < T && idx + 1 < ntiles) {
+      const int gx = se.v.nxp / blockDim.x;
+      const bool wrap = tile.z + 1 == gx;
+      const int ynext = y + (wrap ? (int)blockDim.y : 0);
+      if (ynext < se.v.ny) {
+        const int n1 = (tile.y * se.v.ny + ynext) * se.v.nxp + x + (wrap ? (int)blockDim.x * (1 - gx) : (int)blockDim.x);
+        prefetch_l1(se.v.chunk + (n1 >> 5));
+        prefetch_l1(se.v.flags + n1);
+      }
+    }
+    if (y < se.v.ny) bulk_row<L, S, M, PHYS, true>(se.v, pl, st, x, y, tile.y);
   }
 }
 

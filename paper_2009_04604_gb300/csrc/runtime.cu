@@ -107,7 +107,8 @@ extern "C" int lbm_create(int lattice, const int dims[3], double tau, int dtype,
   if (e == cudaSuccess) e = cudaMalloc(&h->amask, np * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->amask, 0xff, np * sizeof(uint32_t), h->stream);
   if (e == cudaSuccess) e = cudaMalloc(&h->cbase, (np / 32 + 1) * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&h->dres, 8 * sizeof(double));
+  if (e == cudaSuccess) e = cudaHostAlloc(&h->hres, 8 * sizeof(double), cudaHostAllocMapped);
+  if (e == cudaSuccess) e = cudaHostGetDevicePointer(&h->dres, h->hres, 0);
   if (e == cudaSuccess) e = cudaMalloc(&h->err_dev, sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err_dev, 0, sizeof(int), h->stream);
   if (e == cudaSuccess) e = cudaMalloc(&h->dbg_dev, sizeof(unsigned long long));
@@ -194,8 +195,9 @@ int lbm_sim::finish_geometry() {
 }
 
 void lbm_sim::drop_graphs() {
-  for (int k = 0; k < 2; ++k)
-    if (graph[k]) { cudaGraphExecDestroy(graph[k]); graph[k] = nullptr; }
+  for (auto &g : graph)
+    for (int p = 0; p < 2; ++p)
+      if (g[p]) { cudaGraphExecDestroy(g[p]); g[p] = nullptr; }
 }
 
 extern "C" int lbm_destroy(lbm_handle h) {
@@ -204,7 +206,8 @@ extern "C" int lbm_destroy(lbm_handle h) {
   h->drop_graphs();
   h->free_geometry();
   cudaFree(h->f[0]); cudaFree(h->f[1]); cudaFree(h->flags); cudaFree(h->cbase);
-  cudaFree(h->dres); cudaFree(h->scratch); cudaFree(h->tiles); cudaFree(h->err_dev); cudaFree(h->dbg_dev);
+  if (h->hres) cudaFreeHost(h->hres);
+  cudaFree(h->scratch); cudaFree(h->tiles); cudaFree(h->err_dev); cudaFree(h->dbg_dev);
   cudaFree(h->btiles);
   cudaFree(h->amask); cudaFree(h->stage_f); cudaFree(h->dirs);
   h->free_moving_body();
@@ -401,8 +404,9 @@ void lbm_sim::wide_shape() {
 //    blocks for every resident one (256 x 128 x 128 duct, FP16: 82.0 us with one, 80.7
 //    with two; 128 x 96 x 80, FP32: 29.3 and 30.1).
 //  - Register budget: 48 for the bulk kernels of D2Q9 and D3Q19 (D3Q19 duct, FP16: 80.7
-//    us, 83.6 at 64, 84.3 at 40), 64 where they would spill more than a few words (D3Q27,
-//    and a body force under TRT) and for the kernels of the tile table.
+//    us, 83.6 at 64, 84.3 at 40), 64 where they would spill more than a few words (D3Q27
+//    and TRT; D3Q19 TRT duct 100 x 60 x 60, FP32: 12.9 us at 64, 13.6 at 48) and for the
+//    kernels of the tile table.
 void lbm_sim::tune_default() {
   const long long warps = np / 32;
   step_bx = 32;
@@ -414,7 +418,7 @@ void lbm_sim::tune_default() {
   }
   step_by = 4;
   variant = 11;
-  const bool heavy = lattice == LBM_D3Q27 || (has_force && collision == LBM_COLL_TRT);
+  const bool heavy = lattice == LBM_D3Q27 || collision == LBM_COLL_TRT;
   if (!fused() || heavy) variant = 3;
   if (warps >= 4LL * 4 * 152 * 10) tiles_per_block = 2;
 }
@@ -574,8 +578,8 @@ extern "C" int lbm_mass(lbm_handle h, double *m) {
   LBM_CUDA(h, launch_read(h->lattice, h->dtype, h->view(), h->f[h->cur], nullptr, nullptr, nullptr,
                           h->scratch, l));
   LBM_CUDA(h, launch_reduce_final(h->scratch, nblk, 1, h->dres, h->stream));
-  LBM_CUDA(h, cudaMemcpyAsync(m, h->dres, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(h, cudaStreamSynchronize(h->stream));
+  *m = h->hres[0];
   if (!std::isfinite(*m)) return lbm_fail(h, LBM_ERR_NONFINITE, "mass is not finite");
   return LBM_OK;
 }
@@ -607,8 +611,8 @@ extern "C" int lbm_wall_force(lbm_handle h, int tag, double F[3]) {
       LBM_CUDA(h, cudaMemsetAsync(h->scratch + nblk1 * 3, 0, nblk2 * 3 * sizeof(double), h->stream));
   }
   LBM_CUDA(h, launch_reduce_final(h->scratch, nblk1 + nblk2, 3, h->dres, h->stream));
-  LBM_CUDA(h, cudaMemcpyAsync(F, h->dres, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(h, cudaStreamSynchronize(h->stream));
+  std::memcpy(F, h->hres, 3 * sizeof(double));
   return LBM_OK;
 }
 
@@ -628,8 +632,8 @@ extern "C" int lbm_wall_torque(lbm_handle h, int tag, const double centre[3], do
   LBM_CUDA(h, launch_force(h->lattice, h->dtype, v, h->f[h->cur], h->f[h->cur ^ 1], v.stat(), h->nb, nullptr, tag,
                            h->scratch, l, h->scratch + nblk * 3, centre[0], centre[1], centre[2]));
   LBM_CUDA(h, launch_reduce_final(h->scratch + nblk * 3, nblk, 3, h->dres, h->stream));
-  LBM_CUDA(h, cudaMemcpyAsync(T, h->dres, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(h, cudaStreamSynchronize(h->stream));
+  std::memcpy(T, h->hres, 3 * sizeof(double));
   return LBM_OK;
 }
 
@@ -674,41 +678,53 @@ int lbm_sim::launch_steps(int n) {
   return LBM_OK;
 }
 
-int lbm_sim::capture(int parity) {
-  // a graph of kGraphSteps (even) steps starting from buffer `parity`
+int lbm_sim::capture(int k, int parity) {
+  // a graph of kGraphSteps[k] steps starting from buffer `parity`
   const int save = cur;
   cur = parity;
   cudaGraph_t g = nullptr;
   LBM_CUDA(this, cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-  int rc = launch_steps(kGraphSteps);
+  int rc = launch_steps(kGraphSteps[k]);
   cudaError_t e = cudaStreamEndCapture(stream, &g);
   cur = save;
   if (rc) { if (g) cudaGraphDestroy(g); return rc; }
   if (e != cudaSuccess) return lbm_fail(this, LBM_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
-  e = cudaGraphInstantiate(&graph[parity], g, 0);
+  e = cudaGraphInstantiate(&graph[k][parity], g, 0);
   cudaGraphDestroy(g);
-  if (e != cudaSuccess) { graph[parity] = nullptr; return lbm_fail(this, LBM_ERR_CUDA, cudaGetErrorString(e)); }
+  if (e != cudaSuccess) { graph[k][parity] = nullptr; return lbm_fail(this, LBM_ERR_CUDA, cudaGetErrorString(e)); }
   return LBM_OK;
 }
 
+// Steps replay from captured graphs, the longest first. A step of one kernel is as
+// fast launched directly as from a graph of its own, so a remainder of them is. A step
+// of several (boundary tiles forked onto their stream and joined, a body's kernels) is
+// not: a 64 x 32 x 32 FP64 duct takes 106 us a step launched directly, on two streams
+// tied by events, and 50 to 67 from graphs; a step of a 128 x 96 x 80 FP32 duct with its
+// force read back 75 and 65 (with the sum written to the host's memory by the GPU).
 extern "C" int lbm_step(lbm_handle h, int n) {
   if (!h) return lbm_fail(nullptr, LBM_ERR_ARG, "null handle");
   if (n < 0) return lbm_fail(h, LBM_ERR_ARG, "negative step count");
   if (!h->geom_ok || !h->state_ok) return lbm_fail(h, LBM_ERR_STATE, "set geometry and state first");
-  int reps = n / lbm_sim::kGraphSteps;
-  int rest = n % lbm_sim::kGraphSteps;
   if (n > 0) {
     int rc = h->ensure_tiles();  // never inside a capture
     if (rc) return rc;
   }
-  if (reps > 0) {
-    if (!h->graph[h->cur]) {
-      int rc = h->capture(h->cur);
-      if (rc) return rc;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;  // by the caller: no capture of our own inside
+  LBM_CUDA(h, cudaStreamIsCapturing(h->stream, &capturing));
+  const bool single = !h->mb.on && !(h->split() && h->nbtiles > 0);
+  for (int k = 0; k < lbm_sim::kGraphs; ++k) {
+    const int len = lbm_sim::kGraphSteps[k];
+    if (k > 0 && (single || capturing != cudaStreamCaptureStatusNone)) break;
+    for (; n >= len; n -= len) {
+      if (!h->graph[k][h->cur]) {
+        int rc = h->capture(k, h->cur);
+        if (rc) return rc;
+      }
+      LBM_CUDA(h, cudaGraphLaunch(h->graph[k][h->cur], h->stream));
+      h->cur ^= len & 1;
     }
-    for (int k = 0; k < reps; ++k) LBM_CUDA(h, cudaGraphLaunch(h->graph[h->cur], h->stream));
   }
-  return h->launch_steps(rest);
+  return h->launch_steps(n);
 }
 
 // ---------------------------------------------------------------- explicit geometry

@@ -50,7 +50,9 @@ struct MovingBody {
 };
 
 struct lbm_sim {
-  static constexpr int kGraphSteps = 32;  // steps per captured CUDA graph (even)
+  // steps per captured CUDA graph, largest first (a graph of an odd number ends at the other buffer)
+  static constexpr int kGraphs = 3;
+  static constexpr int kGraphSteps[kGraphs] = {32, 8, 1};
 
   int lattice = 0, Q = 9, dtype = 1;
   int nx = 1, ny = 1, nz = 1, nxp = 32;
@@ -86,7 +88,8 @@ struct lbm_sim {
   int has_shell = 0;  // the static geometry has links across thin shells
   unsigned long long geom_hash = 0;  // FNV-1a of the static geometry (flags, records, link data)
 
-  double *dres = nullptr;     // reduction results (device)
+  double *dres = nullptr;     // reduction results: pinned host memory that the GPU writes (hres: the host's view)
+  double *hres = nullptr;
   int *err_dev = nullptr;     // device error word (bit 0: a bounded wait ran out)
   unsigned long long *dbg_dev = nullptr;  // LBM_DEBUG builds: first out-of-range population index
   long long dbg_limit = -1;   // LBM_DEBUG builds: index limit of the checks (-1: Q x padded nodes)
@@ -96,7 +99,7 @@ struct lbm_sim {
   long long wait_limit = 1LL << 24;  // first-wait poll limit of the TMA-staged step
   int refill_mode = 0, refill_iters = 10;  // lbm_set_refill, kept for bodies set later
 
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};  // captured step loops, by starting buffer
+  cudaGraphExec_t graph[kGraphs][2] = {};  // captured step loops, by length and starting buffer
   int2 *tiles = nullptr;      // step-kernel tile table (device)
   long long ntiles = 0;
   int2 *btiles = nullptr;     // split(): the boundary entries (device)
@@ -149,7 +152,7 @@ struct lbm_sim {
   int move_after_step(void *fout, int set);  // body geometry for the next step (geometry.cu)
   int move_rebuild(long long pose);          // body at pose index `pose`, records for f[cur] (geometry.cu)
   void free_moving_body();
-  int capture(int parity);
+  int capture(int k, int parity);
   int upload(const lbm::HostGeometry &g);
   int download(lbm::HostGeometry &g);
   int build_links();      // View::chunk and View::ldesc of the static geometry (geometry.cu)

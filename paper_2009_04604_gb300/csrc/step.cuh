@@ -211,7 +211,7 @@ cudaError_t launch_split_ls(int variant, const View &v, const void *fin, void *f
 template <class Kern>
 cudaError_t batch_kernel(Kern kern, const BatchEntry *e, const int4 *tiles, int n, int T, int parity,
                          const Launch &l) {
-  if (l.smem + (int)(sizeof(BatchEntry) + sizeof(Planes)) > 48 * 1024) {
+  if (l.smem + (int)(sizeof(BatchEntry)) > 48 * 1024) {
     const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, l.smem);
     if (r != cudaSuccess) return r;
   }
