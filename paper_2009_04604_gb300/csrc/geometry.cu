@@ -560,39 +560,36 @@ void exclusive_scan(uint32_t *a, long long n, uint32_t *tot, uint32_t *total, cu
 int lbm_sim::build_links() {
   rplane.assign(nz + 1, 0u);
   if (has_shell) return LBM_OK;  // never fused
-  const long long nchunk = np / 32, nblk = (nchunk + 1023) / 1024;
+  const long long nchunk = np / 32, nblk = (nchunk + 1023) / 1024, pchunks = (long long)nxp * ny / 32;
   const unsigned blocks = (unsigned)((np + 255) / 256);
-  // scratch: open links and packed records before each chunk, the scan's block totals, the two totals
-  uint32_t *obase = nullptr;
+  // scratch (kept by the handle): open links and packed records before each chunk, the
+  // scan's block totals, the total of the open links
+  int rc = ensure_scratch((2 * nchunk + nblk + 4) / 2);
+  if (rc) return rc;
+  uint32_t *obase = reinterpret_cast<uint32_t *>(scratch), *rbase = obase + nchunk, *tot = rbase + nchunk + 1,
+           *total = tot + nblk;
   LBM_CUDA_GEO(this, cudaMalloc(&chunk, nchunk * sizeof(uint4)));
-  LBM_CUDA_GEO(this, cudaMalloc(&obase, (2 * nchunk + nblk + 2) * sizeof(uint32_t)));
-  uint32_t *rbase = obase + nchunk, *tot = rbase + nchunk + 1, *total = tot + nblk;
-  std::vector<uint32_t> hr(nchunk + 1);
   uint32_t nopen = 0;
-  k_geo_lcount<<<blocks, 256, 0, stream>>>(view(), obase, rbase);
-  exclusive_scan(obase, nchunk, tot, total, stream);
-  exclusive_scan(rbase, nchunk, tot, rbase + nchunk, stream);
-  cudaError_t e = cudaMemcpyAsync(&nopen, total, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(hr.data(), rbase, hr.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  if (e == cudaSuccess) {
-    const long long pchunks = (long long)nxp * ny / 32;
+  std::vector<uint32_t> hr(nchunk + 1);
+  if (nb > 0) {
+    k_geo_lcount<<<blocks, 256, 0, stream>>>(view(), obase, rbase);
+    exclusive_scan(obase, nchunk, tot, total, stream);
+    exclusive_scan(rbase, nchunk, tot, rbase + nchunk, stream);
+    LBM_CUDA_GEO(this, cudaMemcpyAsync(&nopen, total, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
+    LBM_CUDA_GEO(this, cudaMemcpyAsync(hr.data(), rbase, hr.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
+    LBM_CUDA_GEO(this, cudaStreamSynchronize(stream));
     for (int z = 0; z <= nz; ++z) rplane[z] = hr[z * pchunks];
-    e = cudaMalloc(&ldesc, std::max<long long>(1, nl + nopen) * sizeof(uint16_t));
+  } else {
+    LBM_CUDA_GEO(this, cudaMemsetAsync(obase, 0, (2 * nchunk + 1) * sizeof(uint32_t), stream));
   }
-  if (e == cudaSuccess && rplane[nz]) e = cudaMalloc(&rrec, rplane[nz] * sizeof(Rec));
-  if (e == cudaSuccess && rplane[nz]) e = cudaMalloc(&rrnode, rplane[nz] * sizeof(uint32_t));
-  if (e == cudaSuccess) {
-    auto *kern = lattice == LBM_D2Q9 ? k_geo_links<D2Q9> : (lattice == LBM_D3Q19 ? k_geo_links<D3Q19> : k_geo_links<D3Q27>);
-    kern<<<blocks, 256, 0, stream>>>(view(), obase, rbase, flags, chunk, ldesc, rrec, rrnode);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  cudaFree(obase);
-  if (e != cudaSuccess)
-    return lbm_fail(this, e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA,
-                    std::string("links by chunk: ") + cudaGetErrorString(e));
+  // one allocation: the packed records, their nodes, the descriptors
+  const size_t nrest = rplane[nz], bytes = nrest * (sizeof(Rec) + sizeof(uint32_t)) + (nl + nopen) * sizeof(uint16_t);
+  if (bytes) LBM_CUDA_GEO(this, cudaMalloc(&rrec, bytes));
+  rrnode = reinterpret_cast<uint32_t *>(rrec + nrest);
+  ldesc = reinterpret_cast<uint16_t *>(rrnode + nrest);
+  auto *kern = lattice == LBM_D2Q9 ? k_geo_links<D2Q9> : (lattice == LBM_D3Q19 ? k_geo_links<D3Q19> : k_geo_links<D3Q27>);
+  kern<<<blocks, 256, 0, stream>>>(view(), obase, rbase, flags, chunk, ldesc, rrec, rrnode);
+  LBM_CUDA_GEO(this, cudaGetLastError());
   return LBM_OK;
 }
 
@@ -889,6 +886,8 @@ __global__ void __launch_bounds__(128) k_move_mark(const MoveGeo g, int refill, 
                                                    uint32_t *__restrict__ crec, uint32_t *__restrict__ clink,
                                                    long long rpad) {
   __shared__ BodyTest b;
+  chain_next();
+  chain_wait();
   load_body(b, g.pose, g.D);
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= rpad) return;  // rpad is a multiple of 32: whole warps
@@ -1037,6 +1036,7 @@ __global__ void __launch_bounds__(kFillThreads) k_move_fill(
   __shared__ double edir[L::Q][3];                  // the same for the directions
   __shared__ uint16_t desc[kFillThreads * (L::Q - 1)];  // thread | direction << 8 of each link
   __shared__ uint32_t wrec[kWarps], wlink[kWarps], base[2], moves[kWarps];
+  chain_wait();
   load_body(bt, g.pose, g.D);
   const GeoShape &b = bt.s;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -1154,6 +1154,8 @@ __global__ void k_body_pose(const MoveGeo g, int koff, int advance, const double
                             double *__restrict__ state, double *__restrict__ hist, int cap, int *__restrict__ step,
                             GeoShape *__restrict__ pose) {
   const int lane = threadIdx.x;
+  chain_next();
+  chain_wait();
   double t = 0.0;
   if (tpart) {
     for (long long b = lane; b < nblk; b += 32) t += tpart[b * 3 + 2];
@@ -1222,8 +1224,11 @@ static cudaError_t move_geometry(lbm_sim *h, int koff, bool after, void *fout, i
   cudaStream_t st = h->stream;
   const unsigned blocks = (unsigned)((mb.rpad + kFillThreads - 1) / kFillThreads);
   const long long nchunk = mb.rpad / 32;
-  k_body_pose<<<1, 32, 0, st>>>(g, koff, after ? 1 : 0, after && mb.free_rot ? mb.tpart : nullptr, mb.nfpart, mb.state,
-                                mb.hist, mb.hist_cap, mb.step, pose);
+  // after a step every kernel of the chain follows the one before it directly (k_force first)
+  cudaError_t e = launch_chained(k_body_pose, dim3(1), dim3(32), 0, st, after, g, koff, after ? 1 : 0,
+                                 after && mb.free_rot ? mb.tpart : nullptr, mb.nfpart, mb.state, mb.hist, mb.hist_cap,
+                                 mb.step, pose);
+  if (e != cudaSuccess) return e;
   return move_dispatch(h->lattice, h->dtype, [&]<class L, typename S, typename M>() {
     const bool lir = after && mb.refill_mode == LBM_REFILL_LIR;
     if (lir) {
@@ -1231,18 +1236,18 @@ static cudaError_t move_geometry(lbm_sim *h, int koff, bool after, void *fout, i
       k_move_lir<L, S, M><<<blocks, kFillThreads, 0, st>>>(g, mb.refill_iters, h->flags, mb.nkind,
                                                            static_cast<S *>(fout));
     }
-    k_move_mark<L, S, M><<<blocks, kFillThreads, 0, st>>>(g, after && !lir ? 1 : 0, h->flags, static_cast<S *>(fout),
-                                                          mb.rcut, mb.crec, mb.clink, mb.rpad);
+    cudaError_t r = launch_chained(k_move_mark<L, S, M>, dim3(blocks), dim3(kFillThreads), 0, st, !lir, g,
+                                   after && !lir ? 1 : 0, h->flags, static_cast<S *>(fout), mb.rcut, mb.crec, mb.clink,
+                                   mb.rpad);
+    if (r != cudaSuccess) return r;
     const bool scan = nchunk > kScanChunks;
     if (scan) {
       exclusive_scan(mb.crec, nchunk, mb.tot, mb.totals, st);
       exclusive_scan(mb.clink, nchunk, mb.tot, mb.totals, st);
     }
-    k_move_fill<L, M><<<blocks, kFillThreads, 0, st>>>(g, mb.rcut, mb.crec, mb.clink, scan, mb.rpad, mb.rec[set],
-                                                       mb.rnode[set], static_cast<M *>(mb.lq[set]),
-                                                       static_cast<M *>(mb.luw[set]), static_cast<M *>(mb.luw1[set]),
-                                                       mb.ltag[set], mb.count[set]);
-    return cudaGetLastError();
+    return launch_chained(k_move_fill<L, M>, dim3(blocks), dim3(kFillThreads), 0, st, !scan, g, mb.rcut, mb.crec,
+                          mb.clink, scan, mb.rpad, mb.rec[set], mb.rnode[set], static_cast<M *>(mb.lq[set]),
+                          static_cast<M *>(mb.luw[set]), static_cast<M *>(mb.luw1[set]), mb.ltag[set], mb.count[set]);
   });
 }
 

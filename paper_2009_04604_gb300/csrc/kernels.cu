@@ -10,6 +10,7 @@ __global__ void k_reduce_final(const double *__restrict__ part, long long nblock
   // 1024 sums took 13 us for three components, this takes 4)
   __shared__ double sm[32];
   const int t = threadIdx.x, lane = t & 31;
+  chain_wait();
   for (int c = 0; c < ncomp; ++c) {
     double s = 0.0;
     for (long long b = t; b < nblocks; b += blockDim.x) s += part[b * ncomp + c];
@@ -29,8 +30,7 @@ cudaError_t launch_reduce_final(const double *part, long long nblocks, int ncomp
                                 cudaStream_t s) {
   // no more warps than there are groups of 32 partials
   const int threads = (int)(nblocks >= 1024 ? 1024 : (nblocks + 31) / 32 * 32);
-  k_reduce_final<<<1, threads > 0 ? threads : 32, 0, s>>>(part, nblocks, ncomp, out);
-  return cudaGetLastError();
+  return launch_chained(k_reduce_final, dim3(1), dim3(threads > 0 ? threads : 32), 0, s, true, part, nblocks, ncomp, out);
 }
 
 // Calls F.template operator()<L, S, M>() for the (lattice, dtype) pair.

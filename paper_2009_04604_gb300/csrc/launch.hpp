@@ -11,8 +11,28 @@ namespace lbm {
 struct Launch {
   dim3 grid, block;
   cudaStream_t stream;
-  int smem = 0;  // dynamic shared memory (TMA-staged step)
+  int smem = 0;  // dynamic shared memory
 };
+
+// A kernel launch that, with chained, may begin while the kernel before it in the stream
+// still runs (programmatic stream serialization): the kernel itself waits, by chain_wait,
+// before it touches what that one reads or writes. Every kernel launched so calls
+// chain_wait first. What it saves is the launch latency between short kernels.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, int smem, cudaStream_t st, bool chained,
+                           A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // Sets the shared-memory limit of the TMA-staged step kernel for this launch shape
 // and returns its persistent grid (SMs x resident blocks, at most ntiles) and its

@@ -144,7 +144,7 @@ extern "C" int lbm_create(int lattice, const int dims[3], double tau, int dtype,
 
 void lbm_sim::free_geometry() {
   cudaFree(rec); cudaFree(rnode); cudaFree(lq); cudaFree(luw); cudaFree(luw1); cudaFree(ltag);
-  cudaFree(chunk); cudaFree(ldesc); cudaFree(rrec); cudaFree(rrnode);
+  cudaFree(chunk); cudaFree(rrec);  // rrnode and ldesc lie behind rrec
   chunk = nullptr; ldesc = nullptr; rrec = nullptr; rrnode = nullptr;
   rec = nullptr; rnode = nullptr; lq = nullptr; luw = nullptr; luw1 = nullptr; ltag = nullptr;
   nb = nl = 0;
