@@ -5,8 +5,9 @@ Workload: the sphere-in-duct configuration at full size. It is a D3Q19 BGK
 outlet and a fixed sphere of radius 16 at (64, 64, 64). Populations are
 stored in FP32, shifted by w_i rho0, and the collision runs in FP32.
 
-One step is one fused stream-collide-boundary pass over the grid: a k_step
-launch, replayed from a CUDA graph. The metric is MLUPS counting fluid nodes,
+One step is one fused stream-collide-boundary pass over the grid, replayed from a
+CUDA graph: the bulk kernel with the walls' boundary kernel beside it, or one
+k_step launch, as the autotuner picks. The metric is MLUPS counting fluid nodes,
 from the best of 5 timed replays of K steps. The roofline fraction divides the
 algorithmic bytes of a launch by its average CUDA-event duration and by the
 measured HBM copy bandwidth. Each of the two population buffers (319 MB) is
@@ -363,14 +364,23 @@ def is_split(tuned):
     return tuned.get("variant") in (9, 10)
 
 
-def step_kernels(tuned):
-    """The kernel(s) of one step at this launch; for the split step the duration is
+def is_bulk(tuned, bc="elibb_f"):
+    """One-node launches under ELIBB-F and -FQ: the bulk tiles and the walls' boundary
+    tiles as two kernels side by side."""
+    return tuned.get("variant") in (0, 1, 2, 3, 11, 12) and bc in ("elibb_f", "elibb_fq")
+
+
+def step_kernels(tuned, bc="elibb_f"):
+    """The kernel(s) of one step at this launch; for two side by side the duration is
     that of the fork-joined pair."""
-    return "k_lattice + k_boundary<D3Q19> (side by side)" if is_split(tuned) else "k_step<D3Q19>"
+    if is_split(tuned):
+        return "k_lattice + k_boundary<D3Q19> (side by side)"
+    return "k_bulk + k_boundary<D3Q19> (side by side)" if is_bulk(tuned, bc) else "k_step<D3Q19>"
 
 
 def profile_name(tuned, dtype, workload):
-    """The committed ncu summary of the step kernel(s) at this launch, dtype and workload."""
+    """The committed ncu summary of the step kernel(s) at this launch, dtype and workload
+    (k_step: the combined and the bulk step)."""
     return f"{'k_lattice_k_boundary' if is_split(tuned) else 'k_step'}_d3q19_{dtype}_{workload}"
 
 
@@ -607,10 +617,10 @@ def ours_arm(args, rank, world, dist):
                      "frac": round(achieved / peak, 4), "traffic": traffic,
                      "peak_source": peak_kind, "algorithmic_bytes_per_launch": int(abytes),
                      "implementation_bytes_per_launch": int(implementation_bytes(nb)),
-                     "kernel": step_kernels(tuned), "duration_us": round(ms_step * 1e3, 2)},
+                     "kernel": step_kernels(tuned, args.bc), "duration_us": round(ms_step * 1e3, 2)},
         "clocks": clk.summary(),
         "e2e": e2e,
-        "gpu_launches": args.steps * REPLAYS * (2 if is_split(tuned) and nb > 0 else 1),
+        "gpu_launches": args.steps * REPLAYS * (2 if (is_split(tuned) or is_bulk(tuned, args.bc)) and nb > 0 else 1),
         "cpu_baseline": cpu,
         "state_finite": finite,
         "accuracy": accuracy,

@@ -250,7 +250,8 @@ int lbm_set_populations(lbm_handle h, const double *f);
 int lbm_get_populations(lbm_handle h, double *f);
 
 /* Enqueue n fused stream-collide-boundary steps on the handle's stream. The
- * steps are replayed from a captured CUDA graph. */
+ * steps are replayed from captured CUDA graphs of 32 steps, and, where a step
+ * takes several kernels, of 8 and 1. */
 int lbm_step(lbm_handle h, int n);
 
 /* Density rho[N] and Guo-corrected velocity u[N*3] ((sum c f + F/2)/rho, Guo
@@ -416,9 +417,10 @@ int lbm_autotune(lbm_handle h, int steps, int *bx, int *by, int *variant, int *t
  * The simulations of a batch share one lattice, one storage type and one stream,
  * and each keeps its own geometry, parameters and state. A batched step runs the
  * same per-node code as lbm_step, so each simulation gets exactly the results it
- * would get alone. The blocks of the launch take the tiles of every simulation
- * (lattice tiles and boundary-record tiles, plane by plane), and the steps replay
- * from captured CUDA graphs. This is for workloads of many small or uneven grids,
+ * would get alone. The blocks of a launch take the tiles of every simulation, and
+ * the steps replay from captured CUDA graphs: per step one launch of the bulk tiles
+ * and, beside it on a stream of the batch, one of the walls' boundary tiles (see
+ * lbm_set_launch; simulations under other rules add a launch of their own). This is for workloads of many small or uneven grids,
  * where one launch per simulation would leave the GPU idle between launches. The
  * handles stay usable on their own; lbm_batch_step picks up their current state. */
 typedef struct lbm_batch_s *lbm_batch;

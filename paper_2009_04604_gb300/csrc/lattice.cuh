@@ -66,14 +66,6 @@ __host__ __device__ constexpr double weight(int i) {
 template <class L>
 __host__ __device__ constexpr int opp(int i) { return L::Q - 1 - i; }
 
-// Threads per block whose boundary work the step kernels stage in static shared
-// memory: 256, or 128 where Q x 256 values of the math type would pass the 48 KB
-// static limit (FP64 on D3Q27). Launches are limited to that many threads.
-template <class L, typename M>
-__host__ __device__ constexpr int stage_threads() {
-  return L::Q * 256 * (int)sizeof(M) <= 48 * 1024 ? 256 : 128;
-}
-
 // Run-time direction index: the velocity components packed as 2-bit fields
 // (component + 1) in 64-bit constants, and the weight in the math type. These
 // keep a rolled loop over links free of lookup chains and of FP64 arithmetic.

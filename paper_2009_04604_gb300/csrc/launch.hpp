@@ -42,14 +42,12 @@ cudaError_t prepare_step_tma(int lattice, int dtype, int phys, int bx, int by, l
                              int *blocks, int *smem);
 
 // lattice: 0 D2Q9, 1 D3Q19, 2 D3Q27; dtype: 0 F64, 1 F32, 2 F16, 3 BF16
-// variant: register budget of the step kernel, at least variant+1 resident
-// 256-thread blocks per SM (0..3), 4: the TMA-staged persistent kernel, 5..7:
-// two nodes per thread with at least 1..3 resident blocks per SM, 8: two nodes
-// per thread in 128-thread blocks, 9 and 10: the split step, whose lattice kernel
-// keeps at least 6 or 5 resident 256-thread blocks per SM and whose boundary
-// kernel runs with the launch lb, 11 and 12: the combined kernel with at least 5
-// or 6 resident 256-thread blocks per SM (FP32/FP16/BF16). FP64 has a single
-// variant.
+// variant: the register budget and form of the step kernel (lbm_set_launch). 0..2: one
+// node per thread at 80 registers, 3: 64, 11: 48, 12: 40, as the bulk step where v.fused,
+// whose boundary kernel runs with the launch lb, else over the tile table; 4: the
+// TMA-staged persistent kernel; 5, 6: two nodes per thread at 128 registers, 7: 80, 8: in
+// 128-thread blocks at 72; 9 and 10: the split step, whose lattice kernel has 40 or 48
+// and whose boundary kernel runs with the launch lb. FP64 has a single budget.
 cudaError_t launch_step(int lattice, int dtype, int variant, const View &v, const void *fin,
                         void *fout, const Launch &l, const Launch *lb = nullptr);
 // One launch of the batched step: n tiles of one kind and physics class (PH_FORCE |

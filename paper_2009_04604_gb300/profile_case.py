@@ -5,7 +5,7 @@
 It builds the workload on the device, steps it W times untimed, then K steps
 per replay (best of R replays, CUDA events on the library's stream), and prints
 one JSON line with the step time and the node, record and link counts. Under
-ncu, `-k regex:k_step -s W+1` skips the warm-up launches. Cases:
+ncu, `-k 'regex:k_bulk|k_boundary' -s 2W` (or `regex:k_step -s W`) skips the warm-up launches. Cases:
 
 - duct:           the sphere duct, D3Q19 256 x 128 x 128, ELIBB-F;
 - box:            the same box, all fluid and periodic (the lattice tiles alone);
