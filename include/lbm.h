@@ -398,7 +398,7 @@ int lbm_set_debug_limit(lbm_handle h, long long elements);
  * The results are the same. Variants 0 and 1 share the register budget of variant 2,
  * variant 5 that of variant 6.
  * Until this call or lbm_autotune the library chooses by size, type and rule: blocks
- * of 32 x 4 nodes (FP64: 32 x 1 or 32 x 2) in variant 11 or 3 (FP64: 0), one
+ * of 32 x 4 nodes (FP64 and D3Q27: also 32 x 1 or 2) in variant 11 or 3 (FP64: 0), one
  * tile per block or, on large lattices, two. lbm_get_launch returns what is in use.
  * LBM_ERR_ARG for an invalid configuration. */
 int lbm_set_launch(lbm_handle h, int bx, int by, int variant, int tiles);

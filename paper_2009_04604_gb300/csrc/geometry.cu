@@ -757,15 +757,6 @@ extern "C" int lbm_build_geometry(lbm_handle h, const uint8_t *base, const doubl
       }
       GEO_CUDA(cudaGetLastError());
     }
-    // fluid node count
-    {
-      std::vector<uint8_t> fl(h->np);
-      GEO_CUDA(cudaMemcpyAsync(fl.data(), h->flags, h->np, cudaMemcpyDeviceToHost, st));
-      GEO_CUDA(cudaStreamSynchronize(st));
-      long long nf = 0;
-      for (long long n = 0; n < h->np; ++n) nf += (fl[n] & 3) == K_FLUID;
-      h->nfluid = nf;
-    }
     rc = h->finish_geometry();
     if (rc) goto done;
     h->geom_ok = true;

@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -22,6 +23,43 @@
 using namespace lbm;
 
 static std::string g_create_error;
+
+// Pinned host memory for the handles' reduction results, which the GPU writes: 64-byte
+// slots of 4 KB pages shared by the process's handles (a page costs more to pin than a
+// handle's device arrays to allocate). The pages go back with the last handle.
+namespace {
+class ResultSlots {
+  std::mutex lock;
+  std::vector<double *> pages, free;
+  size_t used = 0;
+
+ public:
+  cudaError_t take(double **out) {
+    std::lock_guard<std::mutex> guard(lock);
+    if (free.empty()) {
+      double *page = nullptr;
+      cudaError_t e = cudaHostAlloc(&page, 4096, cudaHostAllocMapped | cudaHostAllocPortable);
+      if (e != cudaSuccess) return e;
+      pages.push_back(page);
+      for (int k = 63; k >= 0; --k) free.push_back(page + 8 * k);
+    }
+    *out = free.back();
+    free.pop_back();
+    ++used;
+    return cudaSuccess;
+  }
+  void give(double *p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> guard(lock);
+    free.push_back(p);
+    if (--used > 0) return;
+    for (double *page : pages) cudaFreeHost(page);
+    pages.clear();
+    free.clear();
+  }
+};
+ResultSlots g_results;
+}  // namespace
 
 int lbm_fail(lbm_sim *h, int code, const std::string &msg) {
   if (h) h->err = msg; else g_create_error = msg;
@@ -107,7 +145,7 @@ extern "C" int lbm_create(int lattice, const int dims[3], double tau, int dtype,
   if (e == cudaSuccess) e = cudaMalloc(&h->amask, np * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->amask, 0xff, np * sizeof(uint32_t), h->stream);
   if (e == cudaSuccess) e = cudaMalloc(&h->cbase, (np / 32 + 1) * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaHostAlloc(&h->hres, 8 * sizeof(double), cudaHostAllocMapped);
+  if (e == cudaSuccess) e = g_results.take(&h->hres);
   if (e == cudaSuccess) e = cudaHostGetDevicePointer(&h->dres, h->hres, 0);
   if (e == cudaSuccess) e = cudaMalloc(&h->err_dev, sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->err_dev, 0, sizeof(int), h->stream);
@@ -179,6 +217,8 @@ int lbm_sim::finish_geometry() {
   HostGeometry g;
   int rc = download(g);
   if (rc) return rc;
+  nfluid = 0;
+  for (const uint8_t f : g.flags) nfluid += (f & 3) == K_FLUID;
   if (!launch_set) tune_default();  // thin shells step through the tile table
   unsigned long long h = 0xcbf29ce484222325ULL;
   const long long dims[5] = {lattice, nx, ny, nz, dtype};
@@ -206,7 +246,7 @@ extern "C" int lbm_destroy(lbm_handle h) {
   h->drop_graphs();
   h->free_geometry();
   cudaFree(h->f[0]); cudaFree(h->f[1]); cudaFree(h->flags); cudaFree(h->cbase);
-  if (h->hres) cudaFreeHost(h->hres);
+  g_results.give(h->hres);
   cudaFree(h->scratch); cudaFree(h->tiles); cudaFree(h->err_dev); cudaFree(h->dbg_dev);
   cudaFree(h->btiles);
   cudaFree(h->amask); cudaFree(h->stage_f); cudaFree(h->dirs);
@@ -400,9 +440,11 @@ void lbm_sim::wide_shape() {
 //    35 us a step in 4 blocks of 64 x 4 nodes x 4 tiles, 7.8 in 128 blocks;
 //    64 x 32 x 32 D3Q19: 129 and 50), then two.
 //  - FP32 and below: blocks of 32 x 4 nodes, the best or within 2 % of it at every size
-//    and lattice timed. One tile per block, and two once there are at least four
-//    blocks for every resident one (256 x 128 x 128 duct, FP16: 82.0 us with one, 80.7
-//    with two; 128 x 96 x 80, FP32: 29.3 and 30.1).
+//    timed on D2Q9 and D3Q19. One tile per block, and two on the largest lattices
+//    (256 x 128 x 128 duct, FP16: 82.0 us with one, 80.7 with two; 200 x 100 x 100 47.8
+//    and 48.2, 128 x 96 x 80 in FP32 29.3 and 30.1). D3Q27 takes one warp per block
+//    unless the lattice is small (151 x 67 x 71, FP32: 36.9 us, 45.9 in blocks of 32 x 4;
+//    120 x 80 x 60, FP16: 24.7 and 32.4; 60 x 40 x 40, FP32: 16.7 and 15.5).
 //  - Register budget: 48 for the bulk kernels of D2Q9 and D3Q19 (D3Q19 duct, FP16: 80.7
 //    us, 83.6 at 64, 84.3 at 40), 64 where they would spill more than a few words (D3Q27
 //    and TRT; D3Q19 TRT duct 100 x 60 x 60, FP32: 12.9 us at 64, 13.6 at 48) and for the
@@ -420,7 +462,11 @@ void lbm_sim::tune_default() {
   variant = 11;
   const bool heavy = lattice == LBM_D3Q27 || collision == LBM_COLL_TRT;
   if (!fused() || heavy) variant = 3;
-  if (warps >= 4LL * 4 * 152 * 10) tiles_per_block = 2;
+  if (fused() && lattice == LBM_D3Q27) {
+    if (warps >= 10000) step_by = 1;
+  } else if (warps >= 100000) {
+    tiles_per_block = 2;
+  }
 }
 
 Launch lbm_sim::step_shape() const {
