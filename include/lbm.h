@@ -251,7 +251,8 @@ int lbm_get_populations(lbm_handle h, double *f);
 
 /* Enqueue n fused stream-collide-boundary steps on the handle's stream. The
  * steps are replayed from captured CUDA graphs of 32 steps, and, where a step
- * takes several kernels, of 8 and 1. */
+ * takes several kernels, of 8 and 1. Inside a stream capture of the caller's the
+ * steps are launched one by one into the caller's graph (after one step outside it). */
 int lbm_step(lbm_handle h, int n);
 
 /* Density rho[N] and Guo-corrected velocity u[N*3] ((sum c f + F/2)/rho, Guo

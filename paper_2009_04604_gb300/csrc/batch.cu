@@ -33,6 +33,7 @@ struct lbm_batch_s {
   Range bulk[4], rest[4], boundary;  // tiles by physics class: bulk tiles, the other simulations'; boundary tiles
   cudaStream_t aux = nullptr;        // the boundary tiles' stream, forked and joined around every step
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  cudaStream_t cap = nullptr;        // the stream that steps are captured on
   int bx = 32, by = 4, variant = 3, T = 1;
   bool tiles_ok = false;
   int parity = 0;  // batch steps taken since the entries were built, mod 2
@@ -197,6 +198,30 @@ static int batch_direct(lbm_batch b, int n) {
   return LBM_OK;
 }
 
+// A graph of n steps from parity p, captured on a stream of the batch's own (see lbm_sim::capture).
+static int batch_capture(lbm_batch b, int n, int p, cudaGraphExec_t *out) {
+  if (!b->cap) B_CUDA(b, cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
+  const cudaStream_t user = b->stream;
+  b->stream = b->cap;
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    cudaError_t l = cudaSuccess;
+    for (int k = 0; k < n && l == cudaSuccess; ++k) l = batch_launch(b, (p + k) & 1);
+    e = cudaStreamEndCapture(b->stream, &g);
+    if (l != cudaSuccess) e = l;
+  }
+  b->stream = user;
+  if (e != cudaSuccess) {
+    if (g) cudaGraphDestroy(g);
+    return bfail(b, LBM_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
+  }
+  e = cudaGraphInstantiate(out, g, 0);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) { *out = nullptr; return bfail(b, LBM_ERR_CUDA, cudaGetErrorString(e)); }
+  return LBM_OK;
+}
+
 extern "C" int lbm_batch_create(const lbm_handle *sims, int n, lbm_batch *out) {
   if (!out || !sims || n < 1) return LBM_ERR_ARG;
   *out = nullptr;
@@ -230,6 +255,7 @@ extern "C" int lbm_batch_destroy(lbm_batch b) {
   cudaFree(b->entries);
   cudaFree(b->tiles);
   if (b->aux) { cudaStreamSynchronize(b->aux); cudaStreamDestroy(b->aux); }
+  if (b->cap) cudaStreamDestroy(b->cap);
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   if (b->ev_join) cudaEventDestroy(b->ev_join);
   delete b;
@@ -265,18 +291,15 @@ extern "C" int lbm_batch_step(lbm_batch b, int n) {
     int rc = build_batch(b);
     if (rc) return rc;
   }
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;  // by the caller, into whose graph no other launches
+  B_CUDA(b, cudaStreamIsCapturing(b->stream, &capturing));
+  if (capturing != cudaStreamCaptureStatusNone) return batch_direct(b, n);
   int reps = n / kBatchGraphSteps, rest = n % kBatchGraphSteps;
   if (reps > 0) {
     const int p = b->parity;
     if (!b->graph[p]) {
-      cudaGraph_t g = nullptr;
-      B_CUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-      for (int k = 0; k < kBatchGraphSteps; ++k) batch_launch(b, (p + k) & 1);
-      cudaError_t e = cudaStreamEndCapture(b->stream, &g);
-      if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
-      e = cudaGraphInstantiate(&b->graph[p], g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) { b->graph[p] = nullptr; return bfail(b, LBM_ERR_CUDA, cudaGetErrorString(e)); }
+      int rc = batch_capture(b, kBatchGraphSteps, p, &b->graph[p]);
+      if (rc) return rc;
     }
     for (int k = 0; k < reps; ++k) B_CUDA(b, cudaGraphLaunch(b->graph[p], b->stream));
     // kBatchGraphSteps is even: parities and buffer indices are unchanged

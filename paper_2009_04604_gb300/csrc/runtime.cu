@@ -252,6 +252,7 @@ extern "C" int lbm_destroy(lbm_handle h) {
   cudaFree(h->amask); cudaFree(h->stage_f); cudaFree(h->dirs);
   h->free_moving_body();
   if (h->aux) { cudaStreamSynchronize(h->aux); cudaStreamDestroy(h->aux); }
+  if (h->cap) cudaStreamDestroy(h->cap);
   if (h->ev_fork) cudaEventDestroy(h->ev_fork);
   if (h->ev_join) cudaEventDestroy(h->ev_join);
   if (h->own_stream) cudaStreamDestroy(h->stream);
@@ -724,20 +725,30 @@ int lbm_sim::launch_steps(int n) {
   return LBM_OK;
 }
 
-int lbm_sim::capture(int k, int parity) {
-  // a graph of kGraphSteps[k] steps starting from buffer `parity`
+// A graph of n steps starting from buffer `parity`. The steps are captured on a stream of
+// the handle's own: the caller's may be one that cannot be captured (the legacy stream),
+// one that the caller is capturing, or one that another thread's handle shares, whose
+// launches would land in the graph.
+int lbm_sim::capture(int n, int parity, cudaGraphExec_t *out) {
+  if (!cap) LBM_CUDA(this, cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
   const int save = cur;
+  const cudaStream_t user = stream;
   cur = parity;
+  stream = cap;
   cudaGraph_t g = nullptr;
-  LBM_CUDA(this, cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-  int rc = launch_steps(kGraphSteps[k]);
-  cudaError_t e = cudaStreamEndCapture(stream, &g);
+  cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
+  int rc = LBM_OK;
+  if (e == cudaSuccess) {
+    rc = launch_steps(n);
+    e = cudaStreamEndCapture(stream, &g);
+  }
   cur = save;
+  stream = user;
   if (rc) { if (g) cudaGraphDestroy(g); return rc; }
   if (e != cudaSuccess) return lbm_fail(this, LBM_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
-  e = cudaGraphInstantiate(&graph[k][parity], g, 0);
+  e = cudaGraphInstantiate(out, g, 0);
   cudaGraphDestroy(g);
-  if (e != cudaSuccess) { graph[k][parity] = nullptr; return lbm_fail(this, LBM_ERR_CUDA, cudaGetErrorString(e)); }
+  if (e != cudaSuccess) { *out = nullptr; return lbm_fail(this, LBM_ERR_CUDA, cudaGetErrorString(e)); }
   return LBM_OK;
 }
 
@@ -755,15 +766,16 @@ extern "C" int lbm_step(lbm_handle h, int n) {
     int rc = h->ensure_tiles();  // never inside a capture
     if (rc) return rc;
   }
-  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;  // by the caller: no capture of our own inside
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;  // by the caller, into whose graph no other launches
   LBM_CUDA(h, cudaStreamIsCapturing(h->stream, &capturing));
+  if (capturing != cudaStreamCaptureStatusNone) return h->launch_steps(n);
   const bool single = !h->mb.on && !(h->split() && h->nbtiles > 0);
   for (int k = 0; k < lbm_sim::kGraphs; ++k) {
     const int len = lbm_sim::kGraphSteps[k];
-    if (k > 0 && (single || capturing != cudaStreamCaptureStatusNone)) break;
+    if (k > 0 && single) break;
     for (; n >= len; n -= len) {
       if (!h->graph[k][h->cur]) {
-        int rc = h->capture(k, h->cur);
+        int rc = h->capture(len, h->cur, &h->graph[k][h->cur]);
         if (rc) return rc;
       }
       LBM_CUDA(h, cudaGraphLaunch(h->graph[k][h->cur], h->stream));

@@ -106,6 +106,7 @@ struct lbm_sim {
   long long nbtiles = 0;
   cudaStream_t aux = nullptr;                         // split(): the boundary kernel's stream
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;   // split(): orders aux around each step
+  cudaStream_t cap = nullptr;                         // the stream that steps are captured on
   int tiles_bx = 0, tiles_by = 0;  // launch shape the table was built for (0: stale)
   int tiles_per_block = 4;          // consecutive table entries per step-kernel block (1..4)
   int tiles_var = -1;               // register variant the launch data was prepared for
@@ -152,7 +153,7 @@ struct lbm_sim {
   int move_after_step(void *fout, int set);  // body geometry for the next step (geometry.cu)
   int move_rebuild(long long pose);          // body at pose index `pose`, records for f[cur] (geometry.cu)
   void free_moving_body();
-  int capture(int k, int parity);
+  int capture(int n, int parity, cudaGraphExec_t *out);
   int upload(const lbm::HostGeometry &g);
   int download(lbm::HostGeometry &g);
   int build_links();      // View::chunk and View::ldesc of the static geometry (geometry.cu)
