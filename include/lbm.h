@@ -406,9 +406,10 @@ int lbm_set_launch(lbm_handle h, int bx, int by, int variant, int tiles);
 int lbm_get_launch(lbm_handle h, int *bx, int *by, int *variant, int *tiles);
 
 /* Autotuner: runs `steps` steps with each candidate configuration and keeps the
- * fastest. The candidates are 128- and 256-thread blocks, every admissible bx,
- * every variant with a kernel of its own, and 1, 2 or 4 tiles per block. Each is
- * timed with CUDA events. The simulation advances by every trial step. Writes the chosen
+ * fastest. The candidates are the launch in use, 128- and 256-thread blocks with every
+ * admissible bx and every variant with a kernel of its own, blocks of 32 x 1 and 32 x 2
+ * in variants 0, 3, 11 and 12, and 1, 2 or 4 tiles per block. Each is timed with CUDA
+ * events as lbm_step runs it, replayed from a captured graph. The simulation advances by every trial step. Writes the chosen
  * configuration and its time per step in ms; any output may be NULL.
  * Synchronises the stream. */
 int lbm_autotune(lbm_handle h, int steps, int *bx, int *by, int *variant, int *tiles,

@@ -910,6 +910,29 @@ extern "C" int lbm_get_launch(lbm_handle h, int *bx, int *by, int *variant, int 
   return LBM_OK;
 }
 
+// Time of `steps` steps at the launch in use, as lbm_step runs them: replayed from a graph
+// (at most 32 steps long). A step of two kernels launched directly takes 2 us more on the
+// host than the kernels of a small lattice take on the GPU, so that direct launches rank
+// such lattices by their launches.
+static int time_steps(lbm_sim *h, int steps, cudaEvent_t e0, cudaEvent_t e1, float *ms) {
+  const int len = std::min(steps, lbm_sim::kGraphSteps[0]);
+  cudaGraphExec_t g = nullptr;
+  int rc = h->launch_steps(2);  // warm (and build the tile table)
+  if (rc == LBM_OK) rc = h->capture(len, h->cur, &g);
+  if (rc) return rc;
+  cudaError_t e = cudaGraphUpload(g, h->stream);
+  if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
+  for (int n = steps; n >= len && e == cudaSuccess; n -= len) e = cudaGraphLaunch(g, h->stream);
+  if (e == cudaSuccess && steps <= len) h->cur ^= len & 1;
+  if (e == cudaSuccess) rc = h->launch_steps(steps % len);
+  if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
+  if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+  if (e == cudaSuccess) e = cudaEventElapsedTime(ms, e0, e1);
+  cudaGraphExecDestroy(g);
+  if (e != cudaSuccess) return lbm_fail(h, LBM_ERR_CUDA, cudaGetErrorString(e));
+  return rc;
+}
+
 extern "C" int lbm_autotune(lbm_handle h, int steps, int *bx, int *by, int *variant, int *tiles,
                             double *ms_per_step) {
   if (!h) return lbm_fail(nullptr, LBM_ERR_ARG, "null handle");
@@ -918,47 +941,39 @@ extern "C" int lbm_autotune(lbm_handle h, int steps, int *bx, int *by, int *vari
   cudaEvent_t e0, e1;
   LBM_CUDA(h, cudaEventCreate(&e0));
   LBM_CUDA(h, cudaEventCreate(&e1));
+  h->drop_graphs();
   const int save[4] = {h->step_bx, h->step_by, h->variant, h->tiles_per_block};
   int best[4] = {save[0], save[1], save[2], save[3]};
   float best_ms = 1e30f;
-  int rc = LBM_OK;
+  const auto use = [&](const int *c) {
+    h->step_bx = c[0]; h->step_by = c[1]; h->variant = c[2]; h->tiles_per_block = c[3];
+  };
+  int rc = time_steps(h, steps, e0, e1, &best_ms);  // the launch in use is the one to beat
   const int nvar = h->dtype == LBM_F64 ? 1 : 13;  // 4: TMA; 5-8: node pairs; 9-10: split; 11-12: 5, 6 blocks
   const int tile_opts[3] = {1, 2, 4};
-  for (int threads = 128; threads <= 256 && rc == LBM_OK; threads *= 2)
+  for (int threads = 32; threads <= 256 && rc == LBM_OK; threads *= 2)
     for (int bxx = 32; bxx <= threads && rc == LBM_OK; bxx *= 2) {
       if (h->nxp % bxx) continue;
-      for (int var = 0; var < nvar && rc == LBM_OK; ++var)
+      const bool small = threads < 128;  // blocks of one or two warps: 32 x 1 and 32 x 2 of the one-node kernels
+      if (small && bxx > 32) continue;
+      for (int var = 0; var < nvar && rc == LBM_OK; ++var) {
+        if (var == 1 || var == 2 || var == 6) continue;  // the kernels of 0, 0 and 5
+        if (small && var >= 4 && var <= 10) continue;
         for (int k = 0; k < 3 && rc == LBM_OK; ++k) {
           if (var == 4 && k > 0) continue;  // the persistent kernel ignores tiles per block
-          if (var == 1 || var == 2 || var == 6) continue;  // the kernels of 0, 0 and 5
-          if (!valid_launch(h, bxx, threads / bxx, var, tile_opts[k])) continue;
-          h->step_bx = bxx;
-          h->step_by = threads / bxx;
-          h->variant = var;
-          h->tiles_per_block = tile_opts[k];
-          rc = h->launch_steps(2);  // warm (and build the tile table)
-          if (rc) break;
-          cudaEventRecord(e0, h->stream);
-          rc = h->launch_steps(steps);
-          cudaEventRecord(e1, h->stream);
-          if (rc) break;
-          cudaError_t e = cudaEventSynchronize(e1);
-          if (e != cudaSuccess) { rc = lbm_fail(h, LBM_ERR_CUDA, cudaGetErrorString(e)); break; }
-          float ms = 0.f;
-          cudaEventElapsedTime(&ms, e0, e1);
-          if (ms < best_ms) { best_ms = ms; best[0] = bxx; best[1] = threads / bxx; best[2] = var; best[3] = tile_opts[k]; }
+          const int c[4] = {bxx, threads / bxx, var, tile_opts[k]};
+          if (!valid_launch(h, c[0], c[1], c[2], c[3])) continue;
+          use(c);
+          float ms = 1e30f;
+          rc = time_steps(h, steps, e0, e1, &ms);
+          if (rc == LBM_OK && ms < best_ms) { best_ms = ms; std::copy(c, c + 4, best); }
         }
+      }
     }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (rc) {
-    h->step_bx = save[0]; h->step_by = save[1]; h->variant = save[2]; h->tiles_per_block = save[3];
-    return rc;
-  }
-  h->step_bx = best[0];
-  h->step_by = best[1];
-  h->variant = best[2];
-  h->tiles_per_block = best[3];
+  use(rc ? save : best);
+  if (rc) return rc;
   h->launch_set = true;
   h->drop_graphs();
   if (bx) *bx = best[0];
