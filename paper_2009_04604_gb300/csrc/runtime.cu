@@ -923,7 +923,7 @@ static int time_steps(lbm_sim *h, int steps, cudaEvent_t e0, cudaEvent_t e1, flo
   cudaError_t e = cudaGraphUpload(g, h->stream);
   if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
   for (int n = steps; n >= len && e == cudaSuccess; n -= len) e = cudaGraphLaunch(g, h->stream);
-  if (e == cudaSuccess && steps <= len) h->cur ^= len & 1;
+  if (e == cudaSuccess) h->cur ^= len & 1;  // an odd graph runs once and ends at the other buffer
   if (e == cudaSuccess) rc = h->launch_steps(steps % len);
   if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
   if (e == cudaSuccess) e = cudaEventSynchronize(e1);

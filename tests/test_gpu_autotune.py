@@ -77,3 +77,49 @@ def test_autotune_advances_by_whole_trials(steps):
     s.step(9)
     t.step(9)
     assert np.array_equal(s.get_populations(), t.get_populations())
+
+
+def small_batch(dtype="f32"):
+    import torch
+    st = torch.cuda.Stream()
+    sims = []
+    for dims in [(16, 12, 10), (24, 12, 12)]:
+        base = np.zeros(dims[::-1], np.uint8)
+        base[:, [0, -1]] = lbm.SOLID
+        s = lbm.Simulation(lbm.D3Q19, dims, 0.7, dtype, stream=st)
+        s.set_options("elibb_f", 1.0, (1e-6, 0, 0))
+        s.build_geometry(base.reshape(-1), None, [dict(type="sphere", tag=1, c=(7.6, 5.3, 5.1), r=(2.3, 0, 0))])
+        s.init(1.0)
+        sims.append(s)
+    return sims, lbm.Batch(sims)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_batch_autotune_times_what_runs(dtype):
+    sims, b = small_batch(dtype)
+    class Steps:
+        stream, step = sims[0].stream, staticmethod(b.step)
+    default = step_ms(Steps)
+    got = b.autotune(32)
+    tuned = step_ms(Steps)
+    print(f"default {1e3 * default:.1f} us, tuned {1e3 * tuned:.1f} us, reported {1e3 * got['ms_per_step']:.1f} us", got)
+    assert tuned <= 1.15 * default
+    assert abs(got["ms_per_step"] - tuned) <= 0.25 * tuned
+    b.close()
+
+
+@pytest.mark.parametrize("steps", [1, 7, 32, 71])
+def test_batch_autotune_advances_by_whole_trials(steps):
+    sims, b = small_batch()
+    other, _ = small_batch()
+    b.autotune(steps)
+    want, n = sims[1].get_populations(), 0
+    while not np.array_equal(other[1].get_populations(), want):
+        other[1].step(2 + steps)
+        n += 1
+        assert n < 400
+    assert n > 1
+    b.step(9)
+    other[1].step(9)
+    assert np.array_equal(sims[1].get_populations(), other[1].get_populations())
+    b.close()
