@@ -1470,6 +1470,7 @@ extern "C" int lbm_set_refill(lbm_handle h, int mode, int iterations) {
   if (!h) return lbm_fail(nullptr, LBM_ERR_ARG, "null handle");
   if (mode != LBM_REFILL_EQUILIBRIUM && mode != LBM_REFILL_LIR) return lbm_fail(h, LBM_ERR_ARG, "unknown refill");
   if (iterations < 0 || iterations > 100000) return lbm_fail(h, LBM_ERR_ARG, "iterations must be 0..100000");
+  if (mode == h->refill_mode && iterations == h->refill_iters) return LBM_OK;
   h->refill_mode = mode;
   h->refill_iters = iterations;
   h->mb.refill_mode = mode;

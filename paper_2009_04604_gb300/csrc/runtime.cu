@@ -238,6 +238,7 @@ void lbm_sim::drop_graphs() {
   for (auto &g : graph)
     for (int p = 0; p < 2; ++p)
       if (g[p]) { cudaGraphExecDestroy(g[p]); g[p] = nullptr; }
+  std::fill(asked, asked + kGraphs, 0);
 }
 
 extern "C" int lbm_destroy(lbm_handle h) {
@@ -294,6 +295,9 @@ extern "C" int lbm_set_options(lbm_handle h, int bc, double rho0, const double f
   if (bc == LBM_BC_BFL && h->mb.on)
     return lbm_fail(h, LBM_ERR_ARG, "BFL needs a second node along the link, which a moving body's records do not carry");
   if (!(rho0 > 0.0) || !std::isfinite(rho0)) return lbm_fail(h, LBM_ERR_ARG, "rho0 must be positive");
+  double F[3];
+  for (int a = 0; a < 3; ++a) F[a] = force && !(a == 2 && h->lattice == LBM_D2Q9) ? force[a] : 0.0;
+  if (bc == h->bc && rho0 == h->rho0 && xshift == h->xshift && std::equal(F, F + 3, h->F)) return LBM_OK;
   if (h->geom_ok && h->state_ok && rho0 != h->rho0)
     return lbm_fail(h, LBM_ERR_STATE, "rho0 changes the stored shift: set it before the state");
   if (h->geom_ok && h->state_ok && (bc == LBM_BC_BFL) != (h->bc == LBM_BC_BFL)) {
@@ -314,10 +318,9 @@ extern "C" int lbm_set_options(lbm_handle h, int bc, double rho0, const double f
   h->rho0 = rho0;
   h->has_force = 0;
   for (int a = 0; a < 3; ++a) {
-    h->F[a] = force ? force[a] : 0.0;
-    if (h->F[a] != 0.0) h->has_force = 1;
+    h->F[a] = F[a];
+    if (F[a] != 0.0) h->has_force = 1;
   }
-  if (h->lattice == LBM_D2Q9) { h->F[2] = 0.0; }
   h->xshift = xshift;
   if (!h->launch_set) h->tune_default();
   h->drop_graphs();
@@ -330,6 +333,7 @@ extern "C" int lbm_set_wall_neq(lbm_handle h, int mode) {
   if (!h) return lbm_fail(nullptr, LBM_ERR_ARG, "null handle");
   if (mode != LBM_NEQ_BOUNCE_BACK && mode != LBM_NEQ_REGULARIZED)
     return lbm_fail(h, LBM_ERR_ARG, "unknown wall non-equilibrium estimate");
+  if (mode == h->wall_neq) return LBM_OK;
   h->wall_neq = mode;
   if (!h->launch_set) h->tune_default();
   h->drop_graphs();
@@ -342,6 +346,7 @@ extern "C" int lbm_set_collision(lbm_handle h, int model, double magic) {
   if (model != LBM_COLL_BGK && model != LBM_COLL_TRT) return lbm_fail(h, LBM_ERR_ARG, "unknown collision model");
   if (model == LBM_COLL_TRT && !(magic > 0.0 && std::isfinite(magic)))
     return lbm_fail(h, LBM_ERR_ARG, "the TRT magic parameter must be positive");
+  if (model == h->collision && (model == LBM_COLL_BGK || magic == h->magic)) return LBM_OK;
   h->collision = model;
   if (model == LBM_COLL_TRT) h->magic = magic;
   if (!h->launch_set) h->tune_default();
@@ -758,6 +763,10 @@ int lbm_sim::capture(int n, int parity, cudaGraphExec_t *out) {
 // not: a 64 x 32 x 32 FP64 duct takes 106 us a step launched directly, on two streams
 // tied by events, and 50 to 67 from graphs; a step of a 128 x 96 x 80 FP32 duct with its
 // force read back 75 and 65 (with the sum written to the host's memory by the GPU).
+// Options, geometry and launch changes drop the graphs, so the short ones are captured
+// only when they have been asked for a few times since (kDirectFirst): a capture costs as
+// much as some 60 us of direct launches for 8 steps and 20 for one, and a program that
+// changes the body force before every step would pay it every time.
 extern "C" int lbm_step(lbm_handle h, int n) {
   if (!h) return lbm_fail(nullptr, LBM_ERR_ARG, "null handle");
   if (n < 0) return lbm_fail(h, LBM_ERR_ARG, "negative step count");
@@ -774,6 +783,12 @@ extern "C" int lbm_step(lbm_handle h, int n) {
     const int len = lbm_sim::kGraphSteps[k];
     if (k > 0 && single) break;
     for (; n >= len; n -= len) {
+      if (!h->graph[k][h->cur] && h->asked[k] < lbm_sim::kDirectFirst[k]) {
+        ++h->asked[k];
+        int rc = h->launch_steps(len);
+        if (rc) return rc;
+        continue;
+      }
       if (!h->graph[k][h->cur]) {
         int rc = h->capture(len, h->cur, &h->graph[k][h->cur]);
         if (rc) return rc;

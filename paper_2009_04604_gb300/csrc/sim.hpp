@@ -53,6 +53,7 @@ struct lbm_sim {
   // steps per captured CUDA graph, largest first (a graph of an odd number ends at the other buffer)
   static constexpr int kGraphs = 3;
   static constexpr int kGraphSteps[kGraphs] = {32, 8, 1};
+  static constexpr int kDirectFirst[kGraphs] = {0, 3, 8};  // requests launched directly before a capture
 
   int lattice = 0, Q = 9, dtype = 1;
   int nx = 1, ny = 1, nz = 1, nxp = 32;
@@ -100,6 +101,7 @@ struct lbm_sim {
   int refill_mode = 0, refill_iters = 10;  // lbm_set_refill, kept for bodies set later
 
   cudaGraphExec_t graph[kGraphs][2] = {};  // captured step loops, by length and starting buffer
+  int asked[kGraphs] = {};                 // direct launches in place of each length since drop_graphs
   int2 *tiles = nullptr;      // step-kernel tile table (device)
   long long ntiles = 0;
   int2 *btiles = nullptr;     // split(): the boundary entries (device)
