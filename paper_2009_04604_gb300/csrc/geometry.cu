@@ -552,43 +552,59 @@ static void shape_box(const lbm_shape &s, int D, double lo[3], double hi[3], boo
 
 void exclusive_scan(uint32_t *a, long long n, uint32_t *tot, uint32_t *total, cudaStream_t st) {
   const long long nblk = (n + 1023) / 1024;
-  k_scan_block<<<(unsigned)nblk, 1024, 0, st>>>(a, n, tot);
+  k_scan_block<<<(unsigned)nblk, 1024, 0, st>>>(a, n, nblk == 1 ? total : tot);
+  if (nblk == 1) return;
   k_scan_totals<<<1, 1, 0, st>>>(tot, nblk, total);
   k_scan_add<<<(unsigned)nblk, 1024, 0, st>>>(a, n, tot);
 }
 
-int lbm_sim::build_links() {
-  rplane.assign(nz + 1, 0u);
+// scratch of the two below (kept by the handle): open links and packed records before each
+// chunk, the scan's block totals, the total of the open links
+static void link_scratch(lbm_sim *h, uint32_t *&obase, uint32_t *&rbase, uint32_t *&tot, uint32_t *&total) {
+  const long long nchunk = h->np / 32;
+  obase = reinterpret_cast<uint32_t *>(h->scratch);
+  rbase = obase + nchunk;
+  tot = rbase + nchunk + 1;
+  total = tot + (nchunk + 1023) / 1024;
+}
+
+// before: the packed records before each chunk and in all, in place with nopen once the
+// stream has been waited for (empty without records).
+int lbm_sim::count_links(std::vector<uint32_t> &before) {
+  nopen = 0;
   if (has_shell) return LBM_OK;  // never fused
-  const long long nchunk = np / 32, nblk = (nchunk + 1023) / 1024, pchunks = (long long)nxp * ny / 32;
-  const unsigned blocks = (unsigned)((np + 255) / 256);
-  // scratch (kept by the handle): open links and packed records before each chunk, the
-  // scan's block totals, the total of the open links
+  const long long nchunk = np / 32, nblk = (nchunk + 1023) / 1024;
   int rc = ensure_scratch((2 * nchunk + nblk + 4) / 2);
   if (rc) return rc;
-  uint32_t *obase = reinterpret_cast<uint32_t *>(scratch), *rbase = obase + nchunk, *tot = rbase + nchunk + 1,
-           *total = tot + nblk;
-  LBM_CUDA_GEO(this, cudaMalloc(&chunk, nchunk * sizeof(uint4)));
-  uint32_t nopen = 0;
-  std::vector<uint32_t> hr(nchunk + 1);
-  if (nb > 0) {
-    k_geo_lcount<<<blocks, 256, 0, stream>>>(view(), obase, rbase);
-    exclusive_scan(obase, nchunk, tot, total, stream);
-    exclusive_scan(rbase, nchunk, tot, rbase + nchunk, stream);
-    LBM_CUDA_GEO(this, cudaMemcpyAsync(&nopen, total, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
-    LBM_CUDA_GEO(this, cudaMemcpyAsync(hr.data(), rbase, hr.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
-    LBM_CUDA_GEO(this, cudaStreamSynchronize(stream));
-    for (int z = 0; z <= nz; ++z) rplane[z] = hr[z * pchunks];
-  } else {
+  uint32_t *obase, *rbase, *tot, *total;
+  link_scratch(this, obase, rbase, tot, total);
+  if (nb == 0) {
     LBM_CUDA_GEO(this, cudaMemsetAsync(obase, 0, (2 * nchunk + 1) * sizeof(uint32_t), stream));
+    return LBM_OK;
   }
+  before.resize(nchunk + 1);
+  k_geo_lcount<<<(unsigned)((np + 255) / 256), 256, 0, stream>>>(view(), obase, rbase);
+  exclusive_scan(obase, nchunk, tot, total, stream);
+  exclusive_scan(rbase, nchunk, tot, rbase + nchunk, stream);
+  LBM_CUDA_GEO(this, cudaGetLastError());
+  LBM_CUDA_GEO(this, cudaMemcpyAsync(&nopen, total, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
+  LBM_CUDA_GEO(this, cudaMemcpyAsync(before.data(), rbase, before.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
+  return LBM_OK;
+}
+
+int lbm_sim::build_links(const std::vector<uint32_t> &before) {
+  rplane.assign(nz + 1, 0u);
+  if (has_shell) return LBM_OK;
+  for (int z = 0; z <= nz && !before.empty(); ++z) rplane[z] = before[(long long)z * nxp * ny / 32];
+  uint32_t *obase, *rbase, *tot, *total;
+  link_scratch(this, obase, rbase, tot, total);
   // one allocation: the packed records, their nodes, the descriptors
   const size_t nrest = rplane[nz], bytes = nrest * (sizeof(Rec) + sizeof(uint32_t)) + (nl + nopen) * sizeof(uint16_t);
   if (bytes) LBM_CUDA_GEO(this, cudaMalloc(&rrec, bytes));
   rrnode = reinterpret_cast<uint32_t *>(rrec + nrest);
   ldesc = reinterpret_cast<uint16_t *>(rrnode + nrest);
   auto *kern = lattice == LBM_D2Q9 ? k_geo_links<D2Q9> : (lattice == LBM_D3Q19 ? k_geo_links<D3Q19> : k_geo_links<D3Q27>);
-  kern<<<blocks, 256, 0, stream>>>(view(), obase, rbase, flags, chunk, ldesc, rrec, rrnode);
+  kern<<<(unsigned)((np + 255) / 256), 256, 0, stream>>>(view(), obase, rbase, flags, chunk, ldesc, rrec, rrnode);
   LBM_CUDA_GEO(this, cudaGetLastError());
   return LBM_OK;
 }

@@ -25,8 +25,10 @@ using namespace lbm;
 static std::string g_create_error;
 
 // Pinned host memory for the handles' reduction results, which the GPU writes: 64-byte
-// slots of 4 KB pages shared by the process's handles (a page costs more to pin than a
-// handle's device arrays to allocate). The pages go back with the last handle.
+// slots of 4 KB pages shared by the process's handles. Pinning a page and letting it go
+// costs a lone handle more than its device arrays do (create and destroy, D2Q9 64 x 64:
+// 690 us, 320 with the page kept), so the first page stays with the process. The others go back with
+// the last handle.
 namespace {
 class ResultSlots {
   std::mutex lock;
@@ -34,15 +36,26 @@ class ResultSlots {
   size_t used = 0;
 
  public:
-  cudaError_t take(double **out) {
+  // out: the host's view of a slot, dev: the device's
+  cudaError_t take(double **out, double **dev) {
     std::lock_guard<std::mutex> guard(lock);
+    if (used == 0 && !pages.empty()) {  // the kept page is gone if the device was reset meanwhile
+      void *d = nullptr;
+      if (cudaHostGetDevicePointer(&d, pages[0], 0) != cudaSuccess) {
+        cudaGetLastError();
+        pages.clear();
+        free.clear();
+      }
+    }
     if (free.empty()) {
       double *page = nullptr;
       cudaError_t e = cudaHostAlloc(&page, 4096, cudaHostAllocMapped | cudaHostAllocPortable);
       if (e != cudaSuccess) return e;
       pages.push_back(page);
-      for (int k = 63; k >= 0; --k) free.push_back(page + 8 * k);
+      add(page);
     }
+    cudaError_t e = cudaHostGetDevicePointer(dev, free.back(), 0);
+    if (e != cudaSuccess) return e;
     *out = free.back();
     free.pop_back();
     ++used;
@@ -52,10 +65,16 @@ class ResultSlots {
     if (!p) return;
     std::lock_guard<std::mutex> guard(lock);
     free.push_back(p);
-    if (--used > 0) return;
-    for (double *page : pages) cudaFreeHost(page);
-    pages.clear();
+    if (--used > 0 || pages.size() == 1) return;
+    for (size_t k = 1; k < pages.size(); ++k) cudaFreeHost(pages[k]);
+    pages.resize(1);
     free.clear();
+    add(pages[0]);
+  }
+
+ private:
+  void add(double *page) {
+    for (int k = 63; k >= 0; --k) free.push_back(page + 8 * k);
   }
 };
 ResultSlots g_results;
@@ -141,16 +160,36 @@ extern "C" int lbm_create(int lattice, const int dims[3], double tau, int dtype,
   const size_t bytes = (size_t)h->Q * np * h->elem_size();
   cudaError_t e = cudaMalloc(&h->f[0], bytes);
   if (e == cudaSuccess) e = cudaMalloc(&h->f[1], bytes);
-  if (e == cudaSuccess) e = cudaMalloc(&h->flags, np);
-  if (e == cudaSuccess) e = cudaMalloc(&h->amask, np * sizeof(uint32_t));
+  // One allocation for the small arrays: the directions, the error words, the masks, chunk
+  // words, record counts and kinds of the nodes (each allocation costs as much to make and
+  // to free as a step of a small lattice).
+  const auto up = [](size_t n) { return (n + 255) / 256 * 256; };
+  const size_t at_mask = up(27 * sizeof(LinkDir)) + 256, at_chunk = at_mask + up(np * sizeof(uint32_t)),
+               at_cbase = at_chunk + up(np / 32 * sizeof(uint4)), at_flags = at_cbase + up((np / 32 + 1) * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&h->node_mem, at_flags + np);
+  if (e == cudaSuccess) {
+    unsigned char *m = static_cast<unsigned char *>(h->node_mem);
+    h->dirs = reinterpret_cast<LinkDir *>(m);
+    h->err_dev = reinterpret_cast<int *>(m + at_mask - 256);
+    h->dbg_dev = reinterpret_cast<unsigned long long *>(m + at_mask - 128);
+    h->amask = reinterpret_cast<uint32_t *>(m + at_mask);
+    h->chunk = reinterpret_cast<uint4 *>(m + at_chunk);
+    h->cbase = reinterpret_cast<uint32_t *>(m + at_cbase);
+    h->flags = m + at_flags;
+  }
+  LinkDir dirs[27] = {};
+  {
+    const View v = h->view();
+    for (int i = 0; i < h->Q; ++i) {
+      int c[3];
+      h->lattice_c(i, c[0], c[1], c[2]);
+      dirs[i] = LinkDir{(float)c[0], (float)c[1], (float)c[2], (float)h->lattice_w(i), v.loff[i], {0, 0, 0}};
+    }
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h->dirs, dirs, sizeof(dirs), cudaMemcpyHostToDevice, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->err_dev, 0, 256, h->stream);  // and dbg_dev
   if (e == cudaSuccess) e = cudaMemsetAsync(h->amask, 0xff, np * sizeof(uint32_t), h->stream);
-  if (e == cudaSuccess) e = cudaMalloc(&h->cbase, (np / 32 + 1) * sizeof(uint32_t));
-  if (e == cudaSuccess) e = g_results.take(&h->hres);
-  if (e == cudaSuccess) e = cudaHostGetDevicePointer(&h->dres, h->hres, 0);
-  if (e == cudaSuccess) e = cudaMalloc(&h->err_dev, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->err_dev, 0, sizeof(int), h->stream);
-  if (e == cudaSuccess) e = cudaMalloc(&h->dbg_dev, sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->dbg_dev, 0, sizeof(unsigned long long), h->stream);
+  if (e == cudaSuccess) e = g_results.take(&h->hres, &h->dres);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->flags, K_PAD, np, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->f[0], 0, bytes, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->f[1], 0, bytes, h->stream);
@@ -160,21 +199,6 @@ extern "C" int lbm_create(int lattice, const int dims[3], double tau, int dtype,
     lbm_destroy(h);
     return lbm_fail(nullptr, e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA, msg);
   }
-  {
-    const View v = h->view();
-    LinkDir d[27] = {};
-    for (int i = 0; i < h->Q; ++i) {
-      int c[3];
-      h->lattice_c(i, c[0], c[1], c[2]);
-      d[i] = LinkDir{(float)c[0], (float)c[1], (float)c[2], (float)h->lattice_w(i), v.loff[i], {0, 0, 0}};
-    }
-    e = cudaMalloc(&h->dirs, sizeof(d));
-    if (e == cudaSuccess) e = cudaMemcpy(h->dirs, d, sizeof(d), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      lbm_destroy(h);
-      return lbm_fail(nullptr, e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA, cudaGetErrorString(e));
-    }
-  }
   h->tune_default();
   *out = h;
   return LBM_OK;
@@ -182,8 +206,8 @@ extern "C" int lbm_create(int lattice, const int dims[3], double tau, int dtype,
 
 void lbm_sim::free_geometry() {
   cudaFree(rec); cudaFree(rnode); cudaFree(lq); cudaFree(luw); cudaFree(luw1); cudaFree(ltag);
-  cudaFree(chunk); cudaFree(rrec);  // rrnode and ldesc lie behind rrec
-  chunk = nullptr; ldesc = nullptr; rrec = nullptr; rrnode = nullptr;
+  cudaFree(rrec);  // rrnode and ldesc lie behind rrec
+  ldesc = nullptr; rrec = nullptr; rrnode = nullptr;
   rec = nullptr; rnode = nullptr; lq = nullptr; luw = nullptr; luw1 = nullptr; ltag = nullptr;
   nb = nl = 0;
   has_uw = 0;
@@ -214,8 +238,11 @@ static unsigned long long fnv_words(unsigned long long h, const void *p, size_t 
 // lbm_save / lbm_load).
 int lbm_sim::finish_geometry() {
   LBM_CUDA(this, launch_amask(lattice, view(), amask, stream));
+  std::vector<uint32_t> before;
+  int rc = count_links(before);  // ready with the download
+  if (rc) return rc;
   HostGeometry g;
-  int rc = download(g);
+  rc = download(g);
   if (rc) return rc;
   nfluid = 0;
   for (const uint8_t f : g.flags) nfluid += (f & 3) == K_FLUID;
@@ -231,7 +258,7 @@ int lbm_sim::finish_geometry() {
   h = fnv_words(h, g.luw.data(), g.luw.size());
   h = fnv_words(h, g.luw1.data(), g.luw1.size());
   geom_hash = h;
-  return build_links();  // after the hash: it marks nodes in the flags
+  return build_links(before);  // after the hash: it marks nodes in the flags
 }
 
 void lbm_sim::drop_graphs() {
@@ -246,11 +273,9 @@ extern "C" int lbm_destroy(lbm_handle h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   h->drop_graphs();
   h->free_geometry();
-  cudaFree(h->f[0]); cudaFree(h->f[1]); cudaFree(h->flags); cudaFree(h->cbase);
+  cudaFree(h->f[0]); cudaFree(h->f[1]); cudaFree(h->node_mem);
   g_results.give(h->hres);
-  cudaFree(h->scratch); cudaFree(h->tiles); cudaFree(h->err_dev); cudaFree(h->dbg_dev);
-  cudaFree(h->btiles);
-  cudaFree(h->amask); cudaFree(h->stage_f); cudaFree(h->dirs);
+  cudaFree(h->scratch); cudaFree(h->tiles); cudaFree(h->btiles); cudaFree(h->stage_f);
   h->free_moving_body();
   if (h->aux) { cudaStreamSynchronize(h->aux); cudaStreamDestroy(h->aux); }
   if (h->cap) cudaStreamDestroy(h->cap);

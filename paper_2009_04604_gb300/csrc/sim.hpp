@@ -71,6 +71,7 @@ struct lbm_sim {
 
   void *f[2] = {nullptr, nullptr};  // population buffers; f[cur] holds the current state
   int cur = 0;
+  void *node_mem = nullptr;   // the allocation that holds dirs, err_dev, dbg_dev, amask, chunk, cbase and flags
   uint8_t *flags = nullptr;
   uint32_t *amask = nullptr;  // [np] planes of a non-fluid node that take written-ahead values
   uint32_t *cbase = nullptr;
@@ -84,6 +85,7 @@ struct lbm_sim {
   lbm::Rec *rrec = nullptr;     // the records of the chunks without F_LINKS, for the boundary tiles under fused()
   uint32_t *rrnode = nullptr;
   std::vector<uint32_t> rplane; // [nz + 1] first of them in each plane
+  uint32_t nopen = 0;           // open links
   long long nb = 0, nl = 0, nfluid = 0;
   int has_uw = 0;
   int has_shell = 0;  // the static geometry has links across thin shells
@@ -158,7 +160,8 @@ struct lbm_sim {
   int capture(int n, int parity, cudaGraphExec_t *out);
   int upload(const lbm::HostGeometry &g);
   int download(lbm::HostGeometry &g);
-  int build_links();      // View::chunk and View::ldesc of the static geometry (geometry.cu)
+  int count_links(std::vector<uint32_t> &before);        // nopen, and what rplane is made of (geometry.cu)
+  int build_links(const std::vector<uint32_t> &before);  // rplane, View::chunk and View::ldesc of the static geometry
   int finish_geometry();  // written-ahead masks and hash of the static geometry just set
   int ensure_stage_f();
 };
