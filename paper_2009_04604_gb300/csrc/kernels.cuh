@@ -1665,19 +1665,6 @@ __global__ void k_set_pop(const View v, S *__restrict__ fout, const double *__re
     ST_POP(v, fout, &fout[(long long)i * v.np + n + nb.at(-L::cx(i), -L::cy(i), -L::cz(i))], to_store<S, M>(f[i]));
 }
 
-// A sum kept as an unevaluated pair of floats: h is the rounded sum, l collects the
-// exact rounding errors of every addition (Knuth's TwoSum). About 46 bits.
-struct PairSum {
-  float h = 0.0f, l = 0.0f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
-    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
-    h = s;
-  }
-  __device__ __forceinline__ void sub(float x) { add(-x); }
-  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
-};
-
 // Density and velocity of a node in FP64. The general form sums in FP64.
 template <class L, typename M>
 __device__ __forceinline__ void fields_f64(const View &v, const M (&f)[L::Q], double &r, double (&u)[3]) {
@@ -1696,51 +1683,90 @@ __device__ __forceinline__ void fields_f64(const View &v, const M (&f)[L::Q], do
   for (int a = 0; a < 3; ++a) u[a] = (j[a] + (v.has_force ? 0.5 * v.F[a] : 0.0)) / r;
 }
 
-// The same for FP32 populations, without the FP64 pipe. That pipe issues 2 lanes per
-// clock and SM, 64 times fewer than FP32's, and the 19 conversions, 76 sums and 3
-// divisions a D3Q19 node took there set the kernel's time: 1102 us for the 256 x
-// 128 x 128 duct in FP32, whose bytes take 67; it takes 96 this way. The sums run as PairSum, the quotients
-// as the rounded FP32 quotient and its remainder's, and only the pairs' two halves
-// are added in FP64. Against the FP64 sums the fields differ by less than 1e-13
-// (relative to the density, and to the velocity's largest component). Values outside
-// FP32's comfortable range (and infinities and NaN) take the general form.
+// An FP32 value as a double, on the integer pipe (the conversion takes the FP64 one).
+// Subnormals count as zero.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x);
+  if ((b & 0x7f800000u) == 0u) return 0.0;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// Exact sums of FP32 values on the FP32 pipe, as three floats: every value is cut on a
+// grid common to all, and sums of multiples of the grid's step are exact while they
+// stay below 2^24 steps (Rump, Ogita and Oishi, Accurate floating-point summation, SIAM
+// J. Sci. Comput. 31, 2008). With |f_i| < 2^e, adding and subtracting 1.5 * 2^(e+4)
+// leaves the multiple of 2^(e-19) nearest to f_i, and at most 27 of them add up below
+// 2^(e+5) = 2^24 steps; the remainders, at most 2^(e-20), are cut again at 2^(e-39), and
+// what is left, at most 2^(e-40), is summed as it is, to within 26 * 2^(e-60). That is
+// below 2^-54 sum |f_i|: the FP64 sum's own bound is Q 2^-53 of it.
+struct CutSum {
+  float a = 0.0f, b = 0.0f, c = 0.0f;
+  __device__ __forceinline__ double value() const {
+    double lo = widen(b);
+    if (c != 0.0f) lo += widen(c);  // values below 2^-16 of the node's largest, with bits below 2^-39 of it
+    return widen(a) + lo;
+  }
+};
+
+// The same for FP32 populations, with few FP64 operations. The FP64 pipe issues 2 lanes
+// per clock and SM, 64 times fewer than FP32's, and the 19 conversions, 76 sums and 3
+// divisions that a D3Q19 node took there set the kernel's time: 1102 us for the 256 x
+// 128 x 128 duct in FP32, whose bytes take 67. It takes 171 this way. (Sums as pairs of
+// floats took 109, but hold 46 bits, fewer than FP64's.) The sums are exact in FP32
+// arithmetic (CutSum), the conversions take the integer pipe, and the three quotients
+// share one reciprocal: FP32's, brought to FP64 by one third-order Newton step, and every
+// quotient corrected by its remainder (Markstein, IBM J. Res. Dev. 34, 1990). 17 FP64
+// operations are left. The results are no further from the exact ones than the FP64
+// form's: density and velocity round as its last operations do, and the sums before that
+// are exact. Nodes outside FP32's comfortable range (and infinities and NaN) take the
+// general form; so does a density that cancels to a small part of rho0, for the quotients.
 template <class L>
-__device__ __forceinline__ void fields_pair(const View &v, const ReadPar &rp, const float (&f)[L::Q], double &r,
-                                            double (&u)[3], bool velocity) {
-  PairSum d, j[3];
+__device__ __forceinline__ void fields_f32(const View &v, const ReadPar &rp, const float (&f)[L::Q], double &r,
+                                           double (&u)[3], bool velocity) {
+  uint32_t top = 0u;
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) d.add(f[i]);
-  PairSum rho;
-  rho.h = rp.rho0[0];
-  rho.l = rp.rho0[1];
-  rho.add(d.h);
-  rho.l = __fadd_rn(rho.l, d.l);
-  bool ok = fabsf(rho.h) < 1e30f && fabsf(rho.h) > 1e-30f;
-  if (velocity) {
+  for (int i = 0; i < L::Q; ++i) top = max(top, __float_as_uint(f[i]) & 0x7fffffffu);
+  const uint32_t ex = max(top >> 23, 40u);  // 2^e = 2^(ex - 126)
+  if (ex > 200u || (top != 0u && (top >> 23) < 40u)) {
+    fields_f64<L, float>(v, f, r, u);
+    return;
+  }
+  CutSum d, j[3];
+  const float g1 = __uint_as_float(((ex + 5u) << 23) | 0x400000u), g2 = __uint_as_float(((ex - 15u) << 23) | 0x400000u);
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-      const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
+  for (int i = 0; i < L::Q; ++i) {
+    const float p = __fsub_rn(__fadd_rn(f[i], g1), g1), rest = __fsub_rn(f[i], p);
+    const float q = __fsub_rn(__fadd_rn(rest, g2), g2), w = __fsub_rn(rest, q);
+    d.a = __fadd_rn(d.a, p);
+    d.b = __fadd_rn(d.b, q);
+    d.c = __fadd_rn(d.c, w);
+    const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
-        if (c[a] != 0) {
-          if (c[a] > 0) j[a].add(f[i]); else j[a].sub(f[i]);
-        }
-    }
-    const float inv = __frcp_rn(rho.h);
-#pragma unroll
-    for (int a = 0; a < L::D; ++a) {
-      j[a].add(rp.hF[a][0]);
-      j[a].l = __fadd_rn(j[a].l, rp.hF[a][1]);
-      ok = ok && fabsf(j[a].h) < 1e30f;
-      const float q = __fmul_rn(j[a].h, inv);
-      const float rem = __fmaf_rn(-q, rho.h, j[a].h);  // exact
-      const float rest = __fadd_rn(rem, __fmaf_rn(-q, rho.l, j[a].l));
-      u[a] = (double)q + (double)__fmul_rn(rest, inv);
-    }
-    if (L::D == 2) u[2] = 0.0;
+    for (int k = 0; k < 3; ++k)
+      if (c[k] != 0) {
+        j[k].a = __fadd_rn(j[k].a, c[k] > 0 ? p : -p);
+        j[k].b = __fadd_rn(j[k].b, c[k] > 0 ? q : -q);
+        j[k].c = __fadd_rn(j[k].c, c[k] > 0 ? w : -w);
+      }
   }
   r = v.rho0 + d.value();
-  if (!ok) fields_f64<L, float>(v, f, r, u);
+  if (!velocity) return;
+  const double y0 = widen(__frcp_rn(__fadd_rn(v.rho0_f, __fadd_rn(d.a, d.b))));
+  const double e = __fma_rn(-r, y0, 1.0);
+  const double y = __fma_rn(y0, __fma_rn(e, e, e), y0);  // 1 / r = y0 / (1 - e), to within e^3 of itself
+  const bool near = ((uint32_t)__double2hiint(e) & 0x7fffffffu) < 0x3ed00000u;  // |e| < 2^-18
+#pragma unroll
+  for (int k = 0; k < L::D; ++k) {
+    double m = j[k].value();
+    if (v.has_force) m += rp.hF[k];
+    if (near) {
+      const double q = m * y;
+      u[k] = __fma_rn(__fma_rn(-q, r, m), y, q);
+    } else {
+      u[k] = m / r;
+    }
+  }
+  if (L::D == 2) u[2] = 0.0;
 }
 
 // Pre-collision populations (gathered, BFL-completed), macroscopic fields, and the
@@ -1780,7 +1806,7 @@ __global__ void __launch_bounds__(256) k_read(const __grid_constant__ View v, co
       if (rho_out || u_out || mass_part) {
         double r;
         if constexpr (sizeof(M) == 8) fields_f64<L, M>(v, f, r, u);
-        else fields_pair<L>(v, rp, f, r, u, u_out != nullptr);
+        else fields_f32<L>(v, rp, f, r, u, u_out != nullptr);
         mloc = r;
         if (rho_out) rho_out[hn] = r;
       }

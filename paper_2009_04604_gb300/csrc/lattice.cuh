@@ -264,20 +264,13 @@ template <> struct Par<float> {
         omega_m(v.omega_m_f) {}
 };
 
-// rho0 and half the body force as pairs of floats (their sum is the FP64 value to
-// about 48 bits), for the read-out of FP32 populations (k_read).
+// Half the body force, for the read-out (k_read).
 struct ReadPar {
-  float rho0[2], hF[3][2];
+  double hF[3];
 };
 inline ReadPar read_par(const View &v) {
   ReadPar p;
-  const double val[4] = {v.rho0, v.has_force ? 0.5 * v.F[0] : 0.0, v.has_force ? 0.5 * v.F[1] : 0.0,
-                         v.has_force ? 0.5 * v.F[2] : 0.0};
-  for (int k = 0; k < 4; ++k) {
-    float *o = k == 0 ? p.rho0 : p.hF[k - 1];
-    o[0] = (float)val[k];
-    o[1] = (float)(val[k] - (double)o[0]);
-  }
+  for (int a = 0; a < 3; ++a) p.hF[a] = v.has_force ? 0.5 * v.F[a] : 0.0;
   return p;
 }
 
