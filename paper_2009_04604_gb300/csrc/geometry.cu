@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "lbm.h"
+#include "body_test.hpp"
 #include "geometry.hpp"
 #include "kernels.cuh"
 #include "launch.hpp"
@@ -846,13 +847,12 @@ __device__ __forceinline__ void region_xyz(const MoveGeo &g, long long r, int &x
   z = g.oz + (int)(r / ((long long)g.rx * g.ry));
 }
 
-// A block's copy of the pose, and what decides most solid tests in FP32: the
-// reciprocal semi-axes, the rotation, and a margin around the surface that is far wider
-// than the FP32 error (offsets of a few radii, each rounded once); inside the margin the
-// test is shape_solid's. So the kinds are those of the FP64 definition bit for bit.
+// A block's copy of the pose, and what decides most solid tests in FP32 (body_test.hpp).
+// Inside the margin around the surface the test is shape_solid's, so that the kinds are
+// those of the FP64 definition bit for bit.
 struct BodyTest {
   GeoShape s;
-  float inv[3], ca, sa, tol;
+  BodySurface f;
 };
 
 __device__ __forceinline__ void load_body(BodyTest &b, const GeoShape *__restrict__ pose, int D) {
@@ -862,25 +862,16 @@ __device__ __forceinline__ void load_body(BodyTest &b, const GeoShape *__restric
   __syncthreads();
   if (t == 0) {
     const bool ell = b.s.type == LBM_SHAPE_ELLIPSOID;
-    float rmin = 1e30f;
-    for (int a = 0; a < 3; ++a) {
-      const float r = a < D ? (float)(ell ? b.s.r[a] : b.s.r[0]) : 1.0f;
-      b.inv[a] = 1.0f / r;
-      if (a < D) rmin = fminf(rmin, r);
-    }
-    b.ca = ell ? (float)b.s.ca : 1.0f;
-    b.sa = ell ? (float)b.s.sa : 0.0f;
-    b.tol = 1e-3f * (1.0f + 1.0f / rmin);
+    const double r[3] = {b.s.r[0], ell ? b.s.r[1] : b.s.r[0], ell ? b.s.r[2] : b.s.r[0]};
+    b.f = body_surface(D, r, ell ? b.s.ca : 1.0, ell ? b.s.sa : 0.0);
   }
   __syncthreads();
 }
 
 // d: the FP32 offset of the point x from the body's centre
 __device__ __forceinline__ bool body_solid(const BodyTest &b, int D, float d0, float d1, float d2, int x, int y, int z) {
-  const float t0 = (b.ca * d0 + b.sa * d1) * b.inv[0], t1 = (b.ca * d1 - b.sa * d0) * b.inv[1], t2 = d2 * b.inv[2];
-  const float t = t0 * t0 + t1 * t1 + t2 * t2;
-  if (t < 1.0f - b.tol) return true;
-  if (t > 1.0f + b.tol) return false;
+  const int side = body_side(b.f, d0, d1, d2);
+  if (side != 0) return side > 0;
   return shape_solid(b.s, D, (double)x, (double)y, (double)z);
 }
 
