@@ -125,19 +125,45 @@ def kernel_source_hash():
     return h.hexdigest()[:16]
 
 
-def profiled_traffic(name):
-    """DRAM bytes per launch of a step kernel at the bench's full size, from the
-    committed ncu summary profiles/<name>.json, if it was taken on the current
-    kernel source; else None."""
+def profile_summary(name):
+    """The committed ncu summary profiles/<name>.json if it was taken on the current
+    kernel source, else None."""
     path = os.path.join(ROOT, "profiles", f"{name}.json")
     try:
         with open(path) as fh:
             d = json.load(fh)
         if d.get("kernel_source_hash") == kernel_source_hash():
+            return d
+    except Exception:
+        pass
+    return None
+
+
+def profiled_traffic(name, launch=None):
+    """DRAM bytes per launch of a step kernel at the bench's full size, from its
+    committed summary (profile_summary). With launch (a dict of bx, by, variant, tiles),
+    only if the summary was captured at that launch; else None."""
+    d = profile_summary(name)
+    try:
+        if launch is None or d["launch"] == launch_text(launch):
             return float(d["dram_bytes_per_launch_full_size"])
     except Exception:
         pass
     return None
+
+
+def launch_text(launch):
+    return ",".join(str(launch[k]) for k in ("bx", "by", "variant", "tiles"))
+
+
+def traffic_fields(name, launch):
+    """The traffic of the timed launch, and where only another launch was captured, that
+    one's with the launch it belongs to."""
+    out = {"traffic": profiled_traffic(name, launch)}
+    other = profiled_traffic(name)
+    if out["traffic"] is None and other is not None:
+        out["traffic_of_other_launch"] = {"bytes": other, "launch": profile_summary(name)["launch"]}
+    return out
 
 
 def dist_setup(n):
@@ -270,7 +296,7 @@ def dtype_variant(torch, lbm, W, dtype, steps, peak):
     out = {"value": round(nfluid * steps / (ms * 1e-3) / 1e6, 2), "unit": "MLUPS", "steps": steps,
            "best_of": 5, "ms_per_step": round(ms / steps, 5), "launch": tuned}
     out.update(roofline_of(nfluid, padded_nodes(wl["dims"]), nb, nwall, 19, dtype, False, ms / steps, peak))
-    out["traffic"] = profiled_traffic(profile_name(tuned, dtype, "sphere_duct"))
+    out.update(traffic_fields(profile_name(tuned, dtype, "sphere_duct"), tuned))
     out["kernel"] = step_kernels(tuned)
     return out
 
@@ -300,7 +326,7 @@ def porous_moving(torch, lbm, W, dtype, steps, peak):
            "finite": finite, "ms_per_step": round(ms / steps, 4), "launch": tuned,
            "roofline_note": "static geometry's bytes; the moving sphere's few links add under 0.1 %"}
     out.update(roofline_of(nfluid, padded_nodes(wl["dims"]), nb, nwall, 19, dtype, False, ms / steps, peak))
-    out["traffic"] = profiled_traffic(profile_name(tuned, dtype, "porous_moving"))
+    out.update(traffic_fields(profile_name(tuned, dtype, "porous_moving"), tuned))
     out["kernel"] = step_kernels(tuned)
     return out
 
@@ -351,7 +377,8 @@ def batched_vs_plain(torch, lbm, W, regime, dtype, steps, peak):
                      sum(x[2] for x in c), 19, dtype, False, ms_b / steps, peak)
     out.update({"batched_" + k: v for k, v in rf.items()})
     if regime == "large":
-        out["batched_traffic"] = profiled_traffic(f"k_step_batch_d3q19_{dtype}_batched_ducts")
+        t = traffic_fields(f"k_step_batch_d3q19_{dtype}_batched_ducts", tuned)
+        out.update({"batched_" + k: v for k, v in t.items()})
     return out
 
 
@@ -521,7 +548,7 @@ def ours_arm(args, rank, world, dist):
     ls = 8 if args.dtype == "f64" else 4
     abytes = algorithmic_bytes(nfluid, np_, nb, nwall, 19, s_bytes, ls, False)
     achieved = abytes / (ms_step * 1e-3) / 1e9
-    traffic = profiled_traffic(profile_name(tuned, args.dtype, "sphere_duct"))
+    traffic = traffic_fields(profile_name(tuned, args.dtype, "sphere_duct"), tuned)
     # ---- end to end through the public API: upload the state from pinned host memory,
     # then per step lbm_step(1) and a synchronising read of the drag force (24 B)
     K2 = 1000
@@ -614,7 +641,7 @@ def ours_arm(args, rank, world, dist):
         "mlups_all_nodes": round(world * N * args.steps / (ms * 1e-3) / 1e6, 2),
         "velocity_rel_l2_vs_oracle": accuracy.get(args.dtype, {}).get("velocity_rel_l2_vs_oracle"),
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-                     "frac": round(achieved / peak, 4), "traffic": traffic,
+                     "frac": round(achieved / peak, 4), **traffic,
                      "peak_source": peak_kind, "algorithmic_bytes_per_launch": int(abytes),
                      "implementation_bytes_per_launch": int(implementation_bytes(nb)),
                      "kernel": step_kernels(tuned, args.bc), "duration_us": round(ms_step * 1e3, 2)},
