@@ -1329,7 +1329,7 @@ static int setup_body(lbm_handle h, const lbm_shape *body, const double lo[3], c
   mb.cap_rec = mb.rsize;
   mb.cap_link = mb.rsize * (h->Q - 1);
   mb.tag = body->tag;
-  mb.nfpart = std::min<long long>((mb.cap_rec + 63) / 64, 2 * 152);  // k_force: 8 warps of 8 records a block
+  mb.nfpart = std::min<long long>((mb.cap_rec + 63) / 64, 2 * kSMs);  // k_force: 8 warps of 8 records a block
   GeoShape gs;
   std::memset(&gs, 0, sizeof(gs));
   gs.type = body->type;

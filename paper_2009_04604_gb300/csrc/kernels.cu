@@ -119,7 +119,7 @@ cudaError_t launch_read(int lattice, int dtype, const View &v, const void *fin, 
 static constexpr long long kFewRecords = 5000;
 int force_blocks(long long nrec) {
   const long long per_block = 8 * (nrec <= kFewRecords ? 8 : 32), n = (nrec + per_block - 1) / per_block;
-  return (int)(n < 4 * 152 ? n : 4 * 152);
+  return (int)(n < 4 * kSMs ? n : 4 * kSMs);
 }
 
 cudaError_t launch_force(int lattice, int dtype, const View &v, const void *cur, const void *prev,

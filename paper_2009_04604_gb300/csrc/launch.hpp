@@ -8,6 +8,8 @@
 
 namespace lbm {
 
+constexpr int kSMs = 152;  // of a GB300: the launch rules count warps and blocks per SM
+
 struct Launch {
   dim3 grid, block;
   cudaStream_t stream;

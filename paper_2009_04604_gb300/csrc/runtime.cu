@@ -486,7 +486,7 @@ void lbm_sim::tune_default() {
   tiles_per_block = 1;
   if (dtype == LBM_F64) {
     variant = 0;
-    step_by = warps <= 16 * 152 ? 1 : 2;
+    step_by = warps <= 16 * kSMs ? 1 : 2;
     return;
   }
   step_by = 4;
