@@ -622,7 +622,7 @@ __device__ void boundary(const View &v, const RecSet &rs, const Rec &r, const M 
 // (chain_next), and chain_wait holds them until it is complete and its writes are
 // visible. Both do nothing in a kernel launched the ordinary way. For the chains of
 // short kernels behind a step: k_force and its final sum, a body's kernels (a step and
-// its force read back, 128 x 96 x 80: 65 us before, 63 now). Not for the steps
+// its force read back, 128 x 96 x 80: 2 us less). Not for the steps
 // themselves: alone, a 64 x 64 lattice steps in 7.7 us instead of 8.1, but three such
 // simulations side by side take 5.8 us each instead of 2.9, since the waiting blocks
 // of one stream hold up the others'.
@@ -1888,11 +1888,13 @@ __device__ __noinline__ M shell_outgoing(const View &v, const S *__restrict__ pr
 // point (3 doubles).
 //
 // A warp takes R records at a time and hands their wall links to its lanes, one each.
-// What bounds it is the FP64 pipe (2 lanes per clock and SM): a record per thread ran
-// every direction of the warp's union, at up to 25 FP64 operations each. A link at rest
-// now takes 7: both populations widened, their sum, 2 w rho0, and one addition per
-// component with the velocity's sign. 256 x 128 x 128 duct, 736 thousand links: 42 us
-// before, 18 now; a 128 x 96 x 80 duct 30 and 11. R: launch_force.
+// What bounds it without a tag is the FP64 pipe (2 lanes per clock and SM): a record per
+// thread ran every direction of the warp's union, at up to 25 FP64 operations each. A link
+// at rest now takes 7: both populations widened, their sum, 2 w rho0, and one addition per
+// component with the velocity's sign. With a tag that few links carry, as in a body's drag
+// every step, nearly all links leave at the tag test, and what is left is the walk over
+// the records: loads, ranks and bits. 256 x 128 x 128 duct, 736 thousand links: 18 us, 42
+// with a record per thread; a 128 x 96 x 80 duct 11 and 30. R: launch_force.
 template <class L, typename S, typename M, int R>
 __global__ void __launch_bounds__(256) k_force(const __grid_constant__ View v, const S *__restrict__ cur,
                                                const S *__restrict__ prev, const RecSet rs,

@@ -479,7 +479,11 @@ void lbm_sim::wide_shape() {
 //  - Register budget: 48 for the bulk kernels of D2Q9 and D3Q19 (D3Q19 duct, FP16: 80.7
 //    us, 83.6 at 64, 84.3 at 40), 64 where they would spill more than a few words (D3Q27
 //    and TRT; D3Q19 TRT duct 100 x 60 x 60, FP32: 12.9 us at 64, 13.6 at 48) and for the
-//    kernels of the tile table.
+//    kernels of the tile table (us at 64 registers / 48 / 80, and in wide 256-thread blocks
+//    of four tiles at 80: D3Q19 BFL 128 x 96 x 80 FP32 37.0 / 36.5 / 40.4 and 57.0, 200 x
+//    100 x 100 FP16 TRT 68.5 / 67.1 / 78.6 and 123; D3Q27 BFL 128 x 96 x 80 FP32 60.3 /
+//    66.3 / 59.1 and 101, regularized 64.1 / 70.4 / 59.5 and 86.1; half-way bounce-back
+//    FP16 TRT 50.3 / 66.8 / 52.6 and 85.0).
 void lbm_sim::tune_default() {
   const long long warps = np / 32;
   step_bx = 32;
@@ -785,9 +789,9 @@ int lbm_sim::capture(int n, int parity, cudaGraphExec_t *out) {
 // Steps replay from captured graphs, the longest first. A step of one kernel is as
 // fast launched directly as from a graph of its own, so a remainder of them is. A step
 // of several (boundary tiles forked onto their stream and joined, a body's kernels) is
-// not: a 64 x 32 x 32 FP64 duct takes 106 us a step launched directly, on two streams
-// tied by events, and 50 to 67 from graphs; a step of a 128 x 96 x 80 FP32 duct with its
-// force read back 75 and 65 (with the sum written to the host's memory by the GPU).
+// not always: a 64 x 32 x 32 FP64 duct takes 46 us a step launched directly, on two
+// streams tied by events, 40 from one-step graphs and 36 within a 32-step graph; a step of
+// a 128 x 96 x 80 FP32 duct with its force read back 60 and 57.
 // Options, geometry and launch changes drop the graphs, so the short ones are captured
 // only when they have been asked for a few times since (kDirectFirst): a capture costs as
 // much as some 60 us of direct launches for 8 steps and 20 for one, and a program that
@@ -951,9 +955,8 @@ extern "C" int lbm_get_launch(lbm_handle h, int *bx, int *by, int *variant, int 
 }
 
 // Time of `steps` steps at the launch in use, as lbm_step runs them: replayed from a graph
-// (at most 32 steps long). A step of two kernels launched directly takes 2 us more on the
-// host than the kernels of a small lattice take on the GPU, so that direct launches rank
-// such lattices by their launches.
+// (at most 32 steps long). Timed by direct launches, small lattices are ranked by what the
+// launches cost the host (64 x 48 x 40 FP32: 8.8 us a step, 6.7 from graphs).
 static int time_steps(lbm_sim *h, int steps, cudaEvent_t e0, cudaEvent_t e1, float *ms) {
   const int len = std::min(steps, lbm_sim::kGraphSteps[0]);
   cudaGraphExec_t g = nullptr;
