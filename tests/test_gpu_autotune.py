@@ -52,7 +52,7 @@ CASES = [(lbm.D2Q9, (64, 64, 1), "f64", "bgk"), (lbm.D3Q19, (64, 32, 32), "f64",
 def test_autotune_keeps_the_faster_launch(lat, dims, dtype, collision):
     s = duct(lat, dims, dtype, collision)
     default = step_ms(s)
-    got = s.autotune(10)
+    got = s.autotune(32)
     assert s.get_launch() == (got["bx"], got["by"], got["variant"], got["tiles"])
     tuned = step_ms(s)
     print(f"default {1e3 * default:.1f} us, tuned {1e3 * tuned:.1f} us, reported {1e3 * got['ms_per_step']:.1f} us", got)
