@@ -262,10 +262,12 @@ int lbm_sim::finish_geometry() {
 }
 
 void lbm_sim::drop_graphs() {
-  for (auto &g : graph)
+  for (int k = 0; k < kGraphs; ++k) {
+    if (graph[k][0] || graph[k][1]) lazy[k] = replays[k] < kWorthwhile;
     for (int p = 0; p < 2; ++p)
-      if (g[p]) { cudaGraphExecDestroy(g[p]); g[p] = nullptr; }
-  std::fill(asked, asked + kGraphs, 0);
+      if (graph[k][p]) { cudaGraphExecDestroy(graph[k][p]); graph[k][p] = nullptr; }
+    asked[k] = replays[k] = 0;
+  }
 }
 
 extern "C" int lbm_destroy(lbm_handle h) {
@@ -792,10 +794,14 @@ int lbm_sim::capture(int n, int parity, cudaGraphExec_t *out) {
 // not always: a 64 x 32 x 32 FP64 duct takes 46 us a step launched directly, on two
 // streams tied by events, 40 from one-step graphs and 36 within a 32-step graph; a step of
 // a 128 x 96 x 80 FP32 duct with its force read back 60 and 57.
-// Options, geometry and launch changes drop the graphs, so the short ones are captured
-// only when they have been asked for a few times since (kDirectFirst): a capture costs as
-// much as some 60 us of direct launches for 8 steps and 20 for one, and a program that
-// changes the body force before every step would pay it every time.
+// A capture costs the host some 60 us for 8 steps and 20 for one. While the GPU works on
+// earlier steps of the call that is free, and the short graphs are captured at once (a first
+// pass of 60 steps of the 64 x 32 x 32 FP64 duct takes 3.9 ms so, and 4.9 with its last 28
+// steps launched directly). Otherwise the first requests are launched directly
+// (kDirectFirst: nine steps of a new 64 x 64 FP32 handle 89 us, 120 with captures). Options,
+// geometry and launch changes drop the graphs; where the short ones then had few replays
+// (kWorthwhile), the next wait longer (kLazyFirst), so that a program that changes the body
+// force before every step does not pay a capture each time.
 extern "C" int lbm_step(lbm_handle h, int n) {
   if (!h) return lbm_fail(nullptr, LBM_ERR_ARG, "null handle");
   if (n < 0) return lbm_fail(h, LBM_ERR_ARG, "negative step count");
@@ -808,11 +814,14 @@ extern "C" int lbm_step(lbm_handle h, int n) {
   LBM_CUDA(h, cudaStreamIsCapturing(h->stream, &capturing));
   if (capturing != cudaStreamCaptureStatusNone) return h->launch_steps(n);
   const bool single = !h->mb.on && !(h->split() && h->nbtiles > 0);
+  bool busy = false;  // the GPU has steps of this call to do, so that a capture costs nothing
   for (int k = 0; k < lbm_sim::kGraphs; ++k) {
     const int len = lbm_sim::kGraphSteps[k];
     if (k > 0 && single) break;
     for (; n >= len; n -= len) {
-      if (!h->graph[k][h->cur] && h->asked[k] < lbm_sim::kDirectFirst[k]) {
+      const int direct = h->lazy[k] ? lbm_sim::kLazyFirst[k] : (busy ? 0 : lbm_sim::kDirectFirst[k]);
+      busy = true;
+      if (!h->graph[k][h->cur] && h->asked[k] < direct) {
         ++h->asked[k];
         int rc = h->launch_steps(len);
         if (rc) return rc;
@@ -823,6 +832,7 @@ extern "C" int lbm_step(lbm_handle h, int n) {
         if (rc) return rc;
       }
       LBM_CUDA(h, cudaGraphLaunch(h->graph[k][h->cur], h->stream));
+      if (h->replays[k] < lbm_sim::kWorthwhile) ++h->replays[k];
       h->cur ^= len & 1;
     }
   }

@@ -53,7 +53,9 @@ struct lbm_sim {
   // steps per captured CUDA graph, largest first (a graph of an odd number ends at the other buffer)
   static constexpr int kGraphs = 3;
   static constexpr int kGraphSteps[kGraphs] = {32, 8, 1};
-  static constexpr int kDirectFirst[kGraphs] = {0, 3, 8};  // requests launched directly before a capture
+  static constexpr int kWorthwhile = 4;                    // replays that are worth a capture
+  static constexpr int kDirectFirst[kGraphs] = {0, 1, 2};  // requests launched directly before a capture
+  static constexpr int kLazyFirst[kGraphs] = {0, 3, 8};    // the same where the last captures were in vain
 
   int lattice = 0, Q = 9, dtype = 1;
   int nx = 1, ny = 1, nz = 1, nxp = 32;
@@ -103,7 +105,9 @@ struct lbm_sim {
   int refill_mode = 0, refill_iters = 10;  // lbm_set_refill, kept for bodies set later
 
   cudaGraphExec_t graph[kGraphs][2] = {};  // captured step loops, by length and starting buffer
+  bool lazy[kGraphs] = {};                 // the last graphs of this length were dropped after few replays
   int asked[kGraphs] = {};                 // direct launches in place of each length since drop_graphs
+  int replays[kGraphs] = {};               // launches of each length's graphs since drop_graphs
   int2 *tiles = nullptr;      // step-kernel tile table (device)
   long long ntiles = 0;
   int2 *btiles = nullptr;     // split(): the boundary entries (device)
