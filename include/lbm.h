@@ -407,9 +407,10 @@ int lbm_get_launch(lbm_handle h, int *bx, int *by, int *variant, int *tiles);
 
 /* Autotuner: runs `steps` steps with each candidate configuration and keeps the
  * fastest. The candidates are the launch in use, 128- and 256-thread blocks with every
- * admissible bx and every variant with a kernel of its own, blocks of 32 x 1 and 32 x 2
- * in variants 0, 3, 11 and 12, and 1, 2 or 4 tiles per block. Each is timed with CUDA
- * events as lbm_step runs it, replayed from a captured graph. The simulation advances by every trial step. Writes the chosen
+ * admissible bx and every variant with a kernel of its own, for FP64 and D3Q27 blocks of
+ * 32 x 1 and 32 x 2 in variants 0, 3, 11 and 12, and 1, 2 or 4 tiles per block. Each is
+ * timed with CUDA events by direct launches, and the launch in use and the best of the
+ * others once more as lbm_step runs them, replayed from a captured graph. The simulation advances by every trial step. Writes the chosen
  * configuration and its time per step in ms; any output may be NULL.
  * Synchronises the stream. */
 int lbm_autotune(lbm_handle h, int steps, int *bx, int *by, int *variant, int *tiles,

@@ -964,76 +964,99 @@ extern "C" int lbm_get_launch(lbm_handle h, int *bx, int *by, int *variant, int 
   return LBM_OK;
 }
 
-// Time of `steps` steps at the launch in use, as lbm_step runs them: replayed from a graph
-// (at most 32 steps long). Timed by direct launches, small lattices are ranked by what the
-// launches cost the host (64 x 48 x 40 FP32: 8.8 us a step, 6.7 from graphs).
-static int time_steps(lbm_sim *h, int steps, cudaEvent_t e0, cudaEvent_t e1, float *ms) {
-  const int len = std::min(steps, lbm_sim::kGraphSteps[0]);
+// Time of `steps` steps at the launch in use: launched directly, or as lbm_step runs them,
+// replayed from a graph (at most 32 steps long).
+static int time_steps(lbm_sim *h, int steps, bool graph, cudaEvent_t e0, cudaEvent_t e1, float *ms) {
+  const int len = graph ? std::min(steps, lbm_sim::kGraphSteps[0]) : 1;
   cudaGraphExec_t g = nullptr;
   int rc = h->launch_steps(2);  // warm (and build the tile table)
-  if (rc == LBM_OK) rc = h->capture(len, h->cur, &g);
+  if (rc == LBM_OK && graph) rc = h->capture(len, h->cur, &g);
   if (rc) return rc;
-  cudaError_t e = cudaGraphUpload(g, h->stream);
+  cudaError_t e = graph ? cudaGraphUpload(g, h->stream) : cudaSuccess;
   if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-  for (int n = steps; n >= len && e == cudaSuccess; n -= len) e = cudaGraphLaunch(g, h->stream);
-  if (e == cudaSuccess) h->cur ^= len & 1;  // an odd graph runs once and ends at the other buffer
-  if (e == cudaSuccess) rc = h->launch_steps(steps % len);
+  if (graph) {
+    for (int n = steps; n >= len && e == cudaSuccess; n -= len) e = cudaGraphLaunch(g, h->stream);
+    if (e == cudaSuccess) h->cur ^= len & 1;  // an odd graph runs once and ends at the other buffer
+  }
+  if (e == cudaSuccess) rc = h->launch_steps(graph ? steps % len : steps);
   if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
   if (e == cudaSuccess) e = cudaEventSynchronize(e1);
   if (e == cudaSuccess) e = cudaEventElapsedTime(ms, e0, e1);
-  cudaGraphExecDestroy(g);
+  if (g) cudaGraphExecDestroy(g);
   if (e != cudaSuccess) return lbm_fail(h, LBM_ERR_CUDA, cudaGetErrorString(e));
   return rc;
 }
 
+// Every candidate is timed by direct launches, and the best of them, with the launch in
+// use, once more from a graph, which decides. Direct launches alone rank small lattices by
+// what the launches cost the host (64 x 48 x 40 FP32: 8.8 us a step, 6.7 from graphs), and
+// steps of two kernels, tied across two streams, behind those of one; so the best of either
+// kind are taken, of one kernel only those ahead of all of two. A graph for every candidate would lengthen the tuning of the 256 x 128 x
+// 128 duct by 27 ms.
 extern "C" int lbm_autotune(lbm_handle h, int steps, int *bx, int *by, int *variant, int *tiles,
                             double *ms_per_step) {
   if (!h) return lbm_fail(nullptr, LBM_ERR_ARG, "null handle");
   if (steps < 1) return lbm_fail(h, LBM_ERR_ARG, "steps must be positive");
   if (!h->geom_ok || !h->state_ok) return lbm_fail(h, LBM_ERR_STATE, "set geometry and state first");
+  struct Trial {
+    int bx, by, variant, tiles;
+    float ms;
+  };
+  constexpr size_t kFinalists = 5;  // of either kind
   cudaEvent_t e0, e1;
   LBM_CUDA(h, cudaEventCreate(&e0));
   LBM_CUDA(h, cudaEventCreate(&e1));
   h->drop_graphs();
-  const int save[4] = {h->step_bx, h->step_by, h->variant, h->tiles_per_block};
-  int best[4] = {save[0], save[1], save[2], save[3]};
-  float best_ms = 1e30f;
-  const auto use = [&](const int *c) {
-    h->step_bx = c[0]; h->step_by = c[1]; h->variant = c[2]; h->tiles_per_block = c[3];
+  const Trial saved{h->step_bx, h->step_by, h->variant, h->tiles_per_block, 1e30f};
+  const auto use = [&](const Trial &t) {
+    h->step_bx = t.bx; h->step_by = t.by; h->variant = t.variant; h->tiles_per_block = t.tiles;
   };
-  int rc = time_steps(h, steps, e0, e1, &best_ms);  // the launch in use is the one to beat
+  int rc = LBM_OK;
+  std::vector<Trial> kind[2];  // steps of one kernel, and of two
   const int nvar = h->dtype == LBM_F64 ? 1 : 13;  // 4: TMA; 5-8: node pairs; 9-10: split; 11-12: 5, 6 blocks
   const int tile_opts[3] = {1, 2, 4};
-  for (int threads = 32; threads <= 256 && rc == LBM_OK; threads *= 2)
+  // blocks of one or two warps where the default may be one of them (tune_default)
+  const int least = h->dtype == LBM_F64 || h->lattice == LBM_D3Q27 ? 32 : 128;
+  for (int threads = least; threads <= 256 && rc == LBM_OK; threads *= 2)
     for (int bxx = 32; bxx <= threads && rc == LBM_OK; bxx *= 2) {
       if (h->nxp % bxx) continue;
-      const bool small = threads < 128;  // blocks of one or two warps: 32 x 1 and 32 x 2 of the one-node kernels
+      const bool small = threads < 128;  // 32 x 1 and 32 x 2, of the one-node kernels
       if (small && bxx > 32) continue;
       for (int var = 0; var < nvar && rc == LBM_OK; ++var) {
         if (var == 1 || var == 2 || var == 6) continue;  // the kernels of 0, 0 and 5
         if (small && var >= 4 && var <= 10) continue;
         for (int k = 0; k < 3 && rc == LBM_OK; ++k) {
           if (var == 4 && k > 0) continue;  // the persistent kernel ignores tiles per block
-          const int c[4] = {bxx, threads / bxx, var, tile_opts[k]};
-          if (!valid_launch(h, c[0], c[1], c[2], c[3])) continue;
-          use(c);
-          float ms = 1e30f;
-          rc = time_steps(h, steps, e0, e1, &ms);
-          if (rc == LBM_OK && ms < best_ms) { best_ms = ms; std::copy(c, c + 4, best); }
+          Trial t{bxx, threads / bxx, var, tile_opts[k], 1e30f};
+          if (!valid_launch(h, t.bx, t.by, t.variant, t.tiles)) continue;
+          use(t);
+          rc = time_steps(h, steps, false, e0, e1, &t.ms);
+          kind[h->split() && h->nbtiles > 0].push_back(t);
         }
       }
     }
+  std::vector<Trial> finals{saved};
+  for (auto &c : kind) std::stable_sort(c.begin(), c.end(), [](const Trial &a, const Trial &b) { return a.ms < b.ms; });
+  while (!kind[0].empty() && !kind[1].empty() && kind[0].back().ms > kind[1][0].ms) kind[0].pop_back();
+  for (auto &c : kind) finals.insert(finals.end(), c.begin(), c.begin() + std::min(c.size(), kFinalists));
+  Trial best = saved;
+  for (size_t k = 0; k < finals.size() && rc == LBM_OK; ++k) {
+    Trial t = finals[k];
+    use(t);
+    rc = time_steps(h, steps, true, e0, e1, &t.ms);
+    if (t.ms < best.ms) best = t;
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  use(rc ? save : best);
+  use(rc ? saved : best);
   if (rc) return rc;
   h->launch_set = true;
   h->drop_graphs();
-  if (bx) *bx = best[0];
-  if (by) *by = best[1];
-  if (variant) *variant = best[2];
-  if (tiles) *tiles = best[3];
-  if (ms_per_step) *ms_per_step = best_ms / steps;
+  if (bx) *bx = best.bx;
+  if (by) *by = best.by;
+  if (variant) *variant = best.variant;
+  if (tiles) *tiles = best.tiles;
+  if (ms_per_step) *ms_per_step = best.ms / steps;
   return LBM_OK;
 }
 
